@@ -218,12 +218,10 @@ struct Seg {
     uint32_t rbase;  // cluster rank of the row's first CTA (the fused batch kernel runs several rows per cluster)
 };
 
-// Canonical value of a forward output: from [0, 4q) (Harvey ranges) or [0, 16q) (lazy
-// ranges, reduced to [0, 2q) by a Shoup product with 1 first).
+// Canonical value of a forward output, which the last stage leaves in [0, 4q).
 template <int F>
 __device__ __forceinline__ uint32_t reduce_out(uint32_t x, const LimbConst& lc) {
-    if constexpr ((F & 2) != 0) return csub(mul_shoup_lazy(x, 1u, lc.one_sh, lc.q), lc.q);
-    return csub(csub(x, 2 * lc.q), lc.q);
+    return csub(csub(x, lc.q2), lc.q);
 }
 
 // Loads the 2^R elements jb + k * 2^logs (k < 2^R) of local row `row` into x.
@@ -329,23 +327,55 @@ __device__ __forceinline__ void store_elems(const uint32_t (&x)[1 << R], uint32_
 }
 
 // Lazy-range schedules for moduli below 2^28 (flag F & 2), where values may grow to
-// 16q < 2^32.  A Shoup product with 1 (x - floor(x floor(2^32/q) / 2^32) q, two IMADs)
-// brings any 32-bit value into [0, 2q); it replaces the conditional subtractions of
-// Harvey's butterflies at the few stages where a bound (in units of q) would pass 16.
+// 16q < 2^32.  Bounds are in units of q and brought down by conditional subtractions of 8q, 4q
+// and 2q (an IADD and an unsigned min each), not by a Shoup product with 1: the transforms are
+// bound by the integer-multiply pipe (a Shoup product holds it 8 cycles a warp, a product
+// with 1 for 6), and the adds of a conditional subtraction issue in its shadow.  192 rows of 2^16,
+// with products with 1 / with subtractions: forward 43.1 / 41.7 us, inverse 49.0 / 48.1 us; a
+// batch of 256 uneven products 1171 / 1087 us.
 //  - forward (Cooley-Tukey): the first input enters stage s below fwd_bound_in(s) q; it is
-//    reduced where fwd_bound_in(s) + 2 > 16, and the outputs are below (its bound + 2) q.
-//  - inverse (Gentleman-Sande): both inputs of stage e are below inv_bound_in(e) q (2 for a
-//    canonical or Montgomery-product input); the sum doubles the bound and is reduced where
-//    it would pass 8 (so the next stage's sum and difference stay below 16q).
+//    reduced to 8q where fwd_bound_in(s) + 2 > 16, and the outputs are below (its bound + 2) q.
+//    The transform's last stage reduces it to 2q, so that its outputs are below 4q.
+//  - inverse (Gentleman-Sande): a register pass takes and leaves values below 2q.  Inside it
+//    an element's bound is known from its place: 2 after a product, doubled by each sum since.
+//    A sum that reaches 16 is reduced to 8 before the next stage; the last stage's sums
+//    are reduced to 2.
 __host__ __device__ constexpr int fwd_bound_in(int s) {
     int b = 1;
-    for (int t = 0; t < s; ++t) b = (b + 2 > 16 ? 2 : b) + 2;
+    for (int t = 0; t < s; ++t) b = (b + 2 > 16 ? 8 : b) + 2;
     return b;
 }
-__host__ __device__ constexpr int inv_bound_in(int e) {
+// Bound of element k entering stage v of an inverse register pass (k's bits v-1, v-2, ...: 0 a
+// sum, 1 a product of that stage).
+__host__ __device__ constexpr int inv_bound_in(int v, int k) {
     int b = 2;
-    for (int t = 0; t < e; ++t) b = 2 * b > 8 ? 2 : 2 * b;
+    for (int t = v - 1; t >= 0 && ((k >> t) & 1) == 0; --t) b = 2 * b > 8 ? 8 : 2 * b;
     return b;
+}
+// x below `from` q -> below max(to, ...) q by conditional subtractions (from <= 16; to 2, 4 or 8).
+__device__ __forceinline__ uint32_t reduce_to(uint32_t x, int from, int to, const LimbConst& lc) {
+    if (from > 8 && to <= 8) x = csub(x, lc.q8);
+    if (from > 4 && to <= 4) x = csub(x, lc.q4);
+    if (from > 2 && to <= 2) x = csub(x, lc.q2);
+    return x;
+}
+// Flag bit of F: the forward transform's outputs may be anything below 16q (a Montgomery product
+// follows), so its last stage reduces as any other.
+constexpr int kLooseOut = 64;
+// The first input of forward stage s (of LOGN), brought to where the stage's outputs stay in range.
+template <int LOGN, int F>
+__device__ __forceinline__ uint32_t fwd_first(uint32_t x, int s, const LimbConst& lc) {
+    if constexpr ((F & 2) == 0) return csub(x, lc.q2);
+    const int b = fwd_bound_in(s);
+    if (s == LOGN - 1 && (F & kLooseOut) == 0) return reduce_to(x, b, 2, lc);
+    return b + 2 > 16 ? reduce_to(x, b, 8, lc) : x;
+}
+// The sum of inverse stage v (of R) for element k, brought to where the next stage takes it.
+template <int R, int F>
+__device__ __forceinline__ uint32_t inv_sum(uint32_t sum, int v, int k, const LimbConst& lc) {
+    if constexpr ((F & 2) == 0) return csub(sum, lc.q2);
+    const int b = 2 * inv_bound_in(v, k);
+    return v == R - 1 ? reduce_to(sum, b, 2, lc) : reduce_to(sum, b, 8, lc);
 }
 
 // Twiddle product x w mod q in [0, 2q) for any x < 2^32, by the reduction F selects (bits 2-3):
@@ -366,9 +396,11 @@ __device__ __forceinline__ uint32_t twmul(uint32_t x, uint2 w, const LimbConst& 
     }
 }
 
-// c q for the lazy inverse offsets (c = 2, 4 or 8), from the limb's constants.
-__device__ __forceinline__ uint32_t q_multiple(const LimbConst& lc, int c) {
-    return c == 2 ? lc.q2 : c == 4 ? lc.q4 : c == 8 ? lc.q8 : (uint32_t)c * lc.q;
+// c q with X - Y + c q >= 0 for element k of inverse stage v (Y below c q), from the constants.
+template <int F>
+__device__ __forceinline__ uint32_t inv_offset(const LimbConst& lc, int v, int k) {
+    const int c = (F & 2) != 0 ? inv_bound_in(v, k) : 2;
+    return c == 2 ? lc.q2 : c == 4 ? lc.q4 : lc.q8;
 }
 
 // R forward (Cooley-Tukey) stages s0 .. s0+R-1 on registers; stage s pairs j, j + N/2^(s+1)
@@ -378,12 +410,10 @@ template <int R, int LOGN, int s0, int F>
 __device__ __forceinline__ void fwd_stages(uint32_t (&x)[1 << R], uint32_t g0, const uint2* tw, const LimbConst& lc) {
     // the smallest-stride pass reads the group-major part of the table
     constexpr bool PERM = (s0 + R == LOGN);
-    constexpr bool LAZY = (F & 2) != 0;
-    const uint32_t q = lc.q, two_q = lc.q2;
+    const uint32_t two_q = lc.q2;
 #pragma unroll
     for (int v = 0; v < R; ++v) {
         const int half = 1 << (R - 1 - v);
-        const bool corr = !LAZY || fwd_bound_in(s0 + v) + 2 > 16;
         uint2 w = make_uint2(0, 0);
         // one base pointer per stage: the loads below have compile-time offsets
         const uint2* base = PERM ? tw + g0 + (1u << (s0 + v)) : tw + (1u << (s0 + v)) + ((size_t)g0 << v);
@@ -392,7 +422,7 @@ __device__ __forceinline__ void fwd_stages(uint32_t (&x)[1 << R], uint32_t g0, c
             const int g = b >> (R - 1 - v);
             const int k = (g << (R - v)) + (b & (half - 1));
             if ((b & (half - 1)) == 0) w = __ldg(base + (PERM ? (g << s0) : g));
-            const uint32_t xa = !corr ? x[k] : (LAZY ? mul_shoup_lazy(x[k], 1u, lc.one_sh, q) : csub(x[k], two_q));
+            const uint32_t xa = fwd_first<LOGN, F>(x[k], s0 + v, lc);
             const uint32_t t = twmul<F>(x[k + half], w, lc);
             x[k] = xa + t;
             x[k + half] = xa - t + two_q;
@@ -409,22 +439,18 @@ __device__ __forceinline__ void inv_stages(uint32_t (&x)[1 << R], uint32_t gbase
                                            const LimbConst& lc) {
     constexpr int N = 1 << LOGN;
     constexpr bool PERM = (e0 == 0);  // the smallest-stride pass reads the group-major table part
-    constexpr bool LAZY = (F & 2) != 0;
-    const uint32_t q = lc.q, two_q = lc.q2;
+    const uint32_t q = lc.q;
     const uint32_t J = (gbase >> R) + (uint32_t)j_hi;  // global index of the sub-transform (e0 == 0)
 #pragma unroll
     for (int v = 0; v < R; ++v) {
         const int e = e0 + v;
         const int h = 1 << v;
-        // X - Y + c q >= 0 for Y below c q; the sum is reduced where its bound passes 8q
-        const uint32_t cq = LAZY ? q_multiple(lc, inv_bound_in(e)) : two_q;
-        const bool red = !LAZY || 2 * inv_bound_in(e) > 8;
         if (SCALE && e == LOGN - 1) {
             const uint32_t s = SCALE == 1 ? lc.ninv : lc.ninvR, ssh = SCALE == 1 ? lc.ninv_sh : lc.ninvR_sh;
             const uint32_t w = SCALE == 1 ? lc.ninvw : lc.ninvRw, wsh = SCALE == 1 ? lc.ninvw_sh : lc.ninvRw_sh;
 #pragma unroll
             for (int kk = 0; kk < (1 << (R - 1)); ++kk) {
-                const uint32_t X = x[kk], Y = x[kk + h];
+                const uint32_t X = x[kk], Y = x[kk + h], cq = inv_offset<F>(lc, v, kk);
                 const uint32_t s0v = mul_shoup_lazy(X + Y, s, ssh, q), s1v = mul_shoup_lazy(X - Y + cq, w, wsh, q);
                 x[kk] = csub(s0v, q);
                 x[kk + h] = csub(s1v, q);
@@ -440,9 +466,8 @@ __device__ __forceinline__ void inv_stages(uint32_t (&x)[1 << R], uint32_t gbase
             const int k = (g << (v + 1)) + (b & (h - 1));
             if ((b & (h - 1)) == 0) w = __ldg(base + (PERM ? (g << (LOGN - R)) : g));
             const uint32_t X = x[k], Y = x[k + h];
-            const uint32_t sum = X + Y;
-            x[k] = !red ? sum : (LAZY ? mul_shoup_lazy(sum, 1u, lc.one_sh, q) : csub(sum, two_q));
-            x[k + h] = twmul<F>(X - Y + cq, w, lc);
+            x[k] = inv_sum<R, F>(X + Y, v, k, lc);
+            x[k + h] = twmul<F>(X - Y + inv_offset<F>(lc, v, k), w, lc);
         }
     }
 }
@@ -466,17 +491,15 @@ __device__ __forceinline__ void load_tw_fwd(uint2 (&w)[(1 << R) - 1], uint32_t g
 template <int R, int LOGN, int s0, int F>
 __device__ __forceinline__ void fwd_stages_w(uint32_t (&x)[1 << R], const uint2 (&w)[(1 << R) - 1],
                                              const LimbConst& lc) {
-    constexpr bool LAZY = (F & 2) != 0;
-    const uint32_t q = lc.q, two_q = lc.q2;
+    const uint32_t two_q = lc.q2;
 #pragma unroll
     for (int v = 0; v < R; ++v) {
         const int half = 1 << (R - 1 - v);
-        const bool corr = !LAZY || fwd_bound_in(s0 + v) + 2 > 16;
 #pragma unroll
         for (int b = 0; b < (1 << (R - 1)); ++b) {
             const int g = b >> (R - 1 - v);
             const int k = (g << (R - v)) + (b & (half - 1));
-            const uint32_t xa = !corr ? x[k] : (LAZY ? mul_shoup_lazy(x[k], 1u, lc.one_sh, q) : csub(x[k], two_q));
+            const uint32_t xa = fwd_first<LOGN, F>(x[k], s0 + v, lc);
             const uint32_t t = twmul<F>(x[k + half], w[(1 << v) - 1 + g], lc);
             x[k] = xa + t;
             x[k + half] = xa - t + two_q;
@@ -510,20 +533,17 @@ __device__ __forceinline__ void load_tw_inv(uint2 (&w)[(1 << R) - 1], uint32_t g
 template <int R, int LOGN, int SCALE, int e0, int F>
 __device__ __forceinline__ void inv_stages_w(uint32_t (&x)[1 << R], const uint2 (&w)[(1 << R) - 1],
                                              const LimbConst& lc) {
-    constexpr bool LAZY = (F & 2) != 0;
-    const uint32_t q = lc.q, two_q = lc.q2;
+    const uint32_t q = lc.q;
 #pragma unroll
     for (int v = 0; v < R; ++v) {
         const int e = e0 + v;
         const int h = 1 << v;
-        const uint32_t cq = LAZY ? q_multiple(lc, inv_bound_in(e)) : two_q;
-        const bool red = !LAZY || 2 * inv_bound_in(e) > 8;
         if (SCALE && e == LOGN - 1) {
             const uint32_t s = SCALE == 1 ? lc.ninv : lc.ninvR, ssh = SCALE == 1 ? lc.ninv_sh : lc.ninvR_sh;
             const uint32_t wv = SCALE == 1 ? lc.ninvw : lc.ninvRw, wsh = SCALE == 1 ? lc.ninvw_sh : lc.ninvRw_sh;
 #pragma unroll
             for (int kk = 0; kk < (1 << (R - 1)); ++kk) {
-                const uint32_t X = x[kk], Y = x[kk + h];
+                const uint32_t X = x[kk], Y = x[kk + h], cq = inv_offset<F>(lc, v, kk);
                 const uint32_t s0v = mul_shoup_lazy(X + Y, s, ssh, q), s1v = mul_shoup_lazy(X - Y + cq, wv, wsh, q);
                 x[kk] = csub(s0v, q);
                 x[kk + h] = csub(s1v, q);
@@ -535,9 +555,8 @@ __device__ __forceinline__ void inv_stages_w(uint32_t (&x)[1 << R], const uint2 
             const int g = b >> v;
             const int k = (g << (v + 1)) + (b & (h - 1));
             const uint32_t X = x[k], Y = x[k + h];
-            const uint32_t sum = X + Y;
-            x[k] = !red ? sum : (LAZY ? mul_shoup_lazy(sum, 1u, lc.one_sh, q) : csub(sum, two_q));
-            x[k + h] = twmul<F>(X - Y + cq, w[inv_tw_off(R, v) + g], lc);
+            x[k] = inv_sum<R, F>(X + Y, v, k, lc);
+            x[k + h] = twmul<F>(X - Y + inv_offset<F>(lc, v, k), w[inv_tw_off(R, v) + g], lc);
         }
     }
 }
@@ -725,7 +744,7 @@ __device__ __forceinline__ void fwd_had_inv_pass(uint32_t* sm, const Seg& sg, co
         const LimbConst& lc = row_lc<F>(a, rr);
         uint32_t x[1 << R];
         load_elems<R, LOGN, 0, SRC, F>(x, sm, a, sg, row, jb, lc);
-        fwd_stages<R, LOGN, s0, F>(x, g0, row_twf<N, F>(a, rr), lc);
+        fwd_stages<R, LOGN, s0, F | kLooseOut>(x, g0, row_twf<N, F>(a, rr), lc);
         const bool valid = row < sg.nrows;
         const uint4* hs = reinterpret_cast<const uint4*>(row_had<N, F>(a, valid ? sg.row0 + row : sg.row0) + sg.gbase + jb);
 #pragma unroll
