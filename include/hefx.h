@@ -255,10 +255,10 @@ void hefx_bconv_plan_destroy(hefx_bconv_plan* plan);
  * Results are identical.  The plan has the tensor path when every
  * source prime is below 2^28, L <= 48, Lp <= 64 (one 256-column MMA: four 8-bit chunk
  * columns per target) and the kernel's tiles fit one CTA's shared memory; otherwise
- * HEFX_PATH_TENSOR returns HEFX_EUNSUPPORTED.  HEFX_PATH_AUTO takes the tensor path only when
- * the plan has it, Lp >= 48 and batch * L * n >= 96 * 2^16 (where it measured faster: the
- * CUDA-core kernel makes one pass over the sources per 8 targets, so many targets favour the
- * matrix form); otherwise the CUDA-core path.
+ * HEFX_PATH_TENSOR returns HEFX_EUNSUPPORTED.  HEFX_PATH_AUTO takes the tensor kernel where it
+ * measured faster, sources of 29 and 30 bits included: with more than 8 targets and at least 4
+ * sources, or with up to 8 targets, at least 8 sources, L Lp >= 64 and batch * n >= 2^17
+ * (and N >= 2^7 and tiles that fit); otherwise the CUDA-core path.
  */
 hefx_status hefx_basis_convert(hefx_ctx* ctx, const hefx_bconv_plan* plan, const uint32_t* d_in, uint32_t* d_out,
                                size_t batch, hefx_path path, void* stream);
@@ -283,9 +283,12 @@ hefx_status hefx_bconv_check(hefx_ctx* ctx, const hefx_bconv_plan* plan, void* s
  *                hefx_basis_convert, sources D_j, target limb l of Q u P).
  * hefx_modup_plan_create takes the primes (distinct primes in [3, 2^30), L + K <= 64,
  * alpha in [1, L]) and uploads every digit's constants; EUNSUPPORTED for log2n > 24 or when
- * alpha * max(q) * max(q, p) >= 2^64.  hefx_mod_up converts all digits in one launch on the
- * CUDA cores.  Layouts: d_c [batch][L][N] and d_U [batch][dnum][L + K][N], coefficient form,
- * canonical, 16-byte aligned; d_U must not overlap d_c (EINVAL).
+ * alpha * max(q) * max(q, p) >= 2^64.  hefx_mod_up converts all digits in one launch: as
+ * digit-split matrix products on the tensor cores where that is faster (4 <= alpha <= 48 and the operands
+ * fit a CTA's shared memory), else on the CUDA cores, with the same results.  Layouts: d_c
+ * [batch][L][N] and d_U [batch][dnum][L + K][N], coefficient form, canonical, 16-byte aligned;
+ * d_U must not overlap d_c (EINVAL).  hefx_modup_check waits for `stream` and reports and clears
+ * an expired bounded wait of the plan's launches, as hefx_bconv_check does for conversions.
  */
 hefx_status hefx_modup_plan_create(hefx_ctx* ctx, uint32_t log2n, const uint32_t* q, uint32_t L, const uint32_t* p,
                                    uint32_t K, uint32_t alpha, hefx_modup_plan** out);
@@ -293,6 +296,7 @@ void hefx_modup_plan_destroy(hefx_modup_plan* plan);
 uint32_t hefx_modup_plan_dnum(const hefx_modup_plan* plan); /* 0 for a null plan */
 hefx_status hefx_mod_up(hefx_ctx* ctx, const hefx_modup_plan* plan, const uint32_t* d_c, uint32_t* d_U, size_t batch,
                         void* stream);
+hefx_status hefx_modup_check(hefx_ctx* ctx, const hefx_modup_plan* plan, void* stream);
 
 /*
  * Exact basis conversion (the u-corrected variant of App. B's fast conversion; the paper
@@ -344,7 +348,8 @@ hefx_status hefx_key_inner_product(hefx_ctx* ctx, const hefx_params* params, con
  * where d_x is [batch][L + K][N] in coefficient form (the L ciphertext limbs, then the K
  * special limbs) and d_out is [batch][L][N].  The conversion is the fast one of
  * hefx_basis_convert, so the result represents floor(X / P) - u, 0 <= u < K, for the
- * integer X that d_x represents.  d_out must not overlap d_x.  Runs on the CUDA cores.
+ * integer X that d_x represents.  d_out must not overlap d_x.  Takes the path that
+ * HEFX_PATH_AUTO gives the plan's conversion (hefx_bconv_check reports its waits).
  * Errors: EINVAL for a null, foreign or misaligned argument or overlap.
  */
 hefx_status hefx_mod_down(hefx_ctx* ctx, const hefx_bconv_plan* plan, const uint32_t* d_x, uint32_t* d_out,

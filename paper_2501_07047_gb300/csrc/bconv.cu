@@ -82,7 +82,7 @@ cudaError_t bconv_plan_upload(hefx_bconv_plan* plan) {
     if (e == cudaSuccess) e = cudaMalloc(&plan->d_err, 4);
     if (e == cudaSuccess) e = cudaMemset(plan->d_err, 0, 4);
     if (e != cudaSuccess) return e;
-    return bconv_tc_upload(plan, h);
+    return bconv_tc_create(&h, 1, &plan->tc);
 }
 
 // ModUp of hybrid key switching: digit j (limbs [lo, hi) of Q, alpha per digit) converts to
@@ -102,7 +102,19 @@ cudaError_t modup_plan_upload(hefx_modup_plan* mp) {
     }
     cudaError_t e = cudaMalloc(&mp->d_const, sizeof(BConvConst) * mp->dnum);
     if (e != cudaSuccess) return e;
-    return cudaMemcpy(mp->d_const, h.data(), sizeof(BConvConst) * mp->dnum, cudaMemcpyHostToDevice);
+    e = cudaMemcpy(mp->d_const, h.data(), sizeof(BConvConst) * mp->dnum, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMalloc(&mp->d_err, 4);
+    if (e == cudaSuccess) e = cudaMemset(mp->d_err, 0, 4);
+    return e == cudaSuccess ? bconv_tc_create(h.data(), mp->dnum, &mp->tc) : e;
+}
+
+void modup_plan_free(hefx_modup_plan* mp) {
+    if (mp->d_const) cudaFree(mp->d_const);
+    if (mp->d_err) cudaFree(mp->d_err);
+    bconv_tc_free(mp->tc);
+    mp->d_const = nullptr;
+    mp->d_err = nullptr;
+    mp->tc = nullptr;
 }
 
 void bconv_plan_free(hefx_bconv_plan* plan) {
@@ -110,7 +122,8 @@ void bconv_plan_free(hefx_bconv_plan* plan) {
     plan->d_const = nullptr;
     if (plan->d_err) cudaFree(plan->d_err);
     plan->d_err = nullptr;
-    bconv_tc_free(plan);
+    bconv_tc_free(plan->tc);
+    plan->tc = nullptr;
 }
 
 namespace {
@@ -355,6 +368,8 @@ cudaError_t launch_cc(const hefx_bconv_plan* plan, const uint32_t* in, uint32_t*
 cudaError_t launch_mod_up(const hefx_modup_plan* mp, const uint32_t* c, uint32_t* U, size_t batch,
                           cudaStream_t stream) {
     if (batch == 0) return cudaSuccess;
+    const cudaError_t te = launch_mod_up_tc(mp, c, U, batch, stream);
+    if (te != cudaErrorNotSupported) return te;
     const size_t n = (size_t)1 << mp->log2n;
     const uint32_t rows = mp->L + mp->K;                       // rows of one digit's output
     const uint32_t lp_max = rows - std::min(mp->alpha, mp->L);  // targets of a full digit (the most)
@@ -416,6 +431,8 @@ cudaError_t launch_mod_down(const hefx_bconv_plan* plan, const uint32_t* x, uint
                             cudaStream_t stream) {
     // x: [batch][Lp + L][n] (target-basis limbs first, then the plan's source limbs)
     if (batch == 0) return cudaSuccess;
+    const cudaError_t te = launch_mod_down_tc(plan, x, out, batch, stream);
+    if (te != cudaErrorNotSupported) return te;
     const size_t n = (size_t)1 << plan->log2n;
     return launch_cc<BC_MODDOWN>(plan, x + (size_t)plan->Lp * n, out, x, batch, (size_t)(plan->L + plan->Lp) * n,
                                  stream);

@@ -41,11 +41,10 @@ __device__ __forceinline__ uint32_t barrett64(uint64_t x, uint32_t p, uint64_t m
 // Host: the plan constants of a conversion from src[0..L) to dst[0..Lp) (skip fields 0).
 void fill_bconv_const(const uint32_t* src, uint32_t L, const uint32_t* dst, uint32_t Lp, BConvConst& h);
 
-cudaError_t bconv_tc_upload(hefx_bconv_plan* plan, const BConvConst& h);
-void bconv_tc_free(hefx_bconv_plan* plan);
+cudaError_t bconv_tc_create(const BConvConst* h, uint32_t count, BcTcPlan** out);
+void bconv_tc_free(BcTcPlan* tp);
 bool bconv_tc_available(const hefx_bconv_plan* plan);
-// The path HEFX_PATH_AUTO takes for a call of `batch` polynomials (measured rule: the tensor
-// path wins only with more than 8 targets on throughput-sized calls).
+// The path HEFX_PATH_AUTO takes for a call of `batch` polynomials.
 bool bconv_prefer_tc(const hefx_bconv_plan* plan, size_t batch);
 
 }  // namespace hefx

@@ -534,7 +534,7 @@ hefx_status hefx_modup_plan_create(hefx_ctx* ctx, uint32_t log2n, const uint32_t
 
 void hefx_modup_plan_destroy(hefx_modup_plan* mp) {
     if (!mp) return;
-    if (mp->d_const) cudaFree(mp->d_const);
+    modup_plan_free(mp);
     delete mp;
 }
 
@@ -569,9 +569,9 @@ hefx_status hefx_basis_convert(hefx_ctx* ctx, const hefx_bconv_plan* plan, const
         return fail(ctx, HEFX_EINVAL, "d_out overlaps d_in");
     hefx_status st = use_device(ctx);
     if (st != HEFX_OK) return st;
-    if (path == HEFX_PATH_AUTO) path = bconv_prefer_tc(plan, batch) ? HEFX_PATH_TENSOR : HEFX_PATH_CUDACORE;
-    if (path == HEFX_PATH_TENSOR && !bconv_tc_available(plan))
+    if (path == HEFX_PATH_TENSOR && !bconv_tc_available(plan))  // an explicit request; AUTO has its own rule
         return fail(ctx, HEFX_EUNSUPPORTED, "tensor basis conversion not available for this plan");
+    if (path == HEFX_PATH_AUTO) path = bconv_prefer_tc(plan, batch) ? HEFX_PATH_TENSOR : HEFX_PATH_CUDACORE;
     if (batch == 0) return HEFX_OK;
     cudaError_t e;
     if (path == HEFX_PATH_TENSOR)
@@ -586,22 +586,33 @@ hefx_status hefx_basis_convert(hefx_ctx* ctx, const hefx_bconv_plan* plan, const
     return HEFX_OK;
 }
 
-hefx_status hefx_bconv_check(hefx_ctx* ctx, const hefx_bconv_plan* plan, void* stream) {
-    if (!ctx) return HEFX_EINVAL;
-    if (!plan || plan->ctx != ctx) return fail(ctx, HEFX_EINVAL, "plan is null or belongs to another context");
+// Reports and clears a conversion plan's bounded-wait flag, after the stream's work.
+static hefx_status conversion_check(hefx_ctx* ctx, uint32_t* d_err, void* stream, const char* name) {
     hefx_status st = use_device(ctx);
     if (st != HEFX_OK) return st;
     uint32_t code = 0;
     cudaError_t e = cudaSuccess;
-    if (plan->d_err) {
-        e = cudaMemcpyAsync(&code, plan->d_err, 4, cudaMemcpyDeviceToHost, (cudaStream_t)stream);
+    if (d_err) {
+        e = cudaMemcpyAsync(&code, d_err, 4, cudaMemcpyDeviceToHost, (cudaStream_t)stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize((cudaStream_t)stream);
-        if (e == cudaSuccess && code) e = cudaMemsetAsync(plan->d_err, 0, 4, (cudaStream_t)stream);
+        if (e == cudaSuccess && code) e = cudaMemsetAsync(d_err, 0, 4, (cudaStream_t)stream);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize((cudaStream_t)stream);
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "hefx_bconv_check");
+    if (e != cudaSuccess) return cuda_fail(ctx, e, name);
     if (code) return fail(ctx, HEFX_ETIMEOUT, "a bounded device wait of a basis conversion expired (code %u); results are invalid", code);
     return HEFX_OK;
+}
+
+hefx_status hefx_bconv_check(hefx_ctx* ctx, const hefx_bconv_plan* plan, void* stream) {
+    if (!ctx) return HEFX_EINVAL;
+    if (!plan || plan->ctx != ctx) return fail(ctx, HEFX_EINVAL, "plan is null or belongs to another context");
+    return conversion_check(ctx, plan->d_err, stream, "hefx_bconv_check");
+}
+
+hefx_status hefx_modup_check(hefx_ctx* ctx, const hefx_modup_plan* plan, void* stream) {
+    if (!ctx) return HEFX_EINVAL;
+    if (!plan || plan->ctx != ctx) return fail(ctx, HEFX_EINVAL, "plan is null or belongs to another context");
+    return conversion_check(ctx, plan->d_err, stream, "hefx_modup_check");
 }
 
 hefx_status hefx_basis_convert_exact(hefx_ctx* ctx, const hefx_bconv_plan* plan, const uint32_t* in, uint32_t* out,

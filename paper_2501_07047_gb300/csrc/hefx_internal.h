@@ -63,6 +63,7 @@ struct BcListEntry {
     const uint32_t* in;
     uint32_t* out;
 };
+struct BcTcPlan;  // tensor form of a plan's conversions (bconv_tc.cu)
 
 // One cluster task of the fused batch kernel (ntt_cc_batch.cu): nrows rows of ring degree
 // 2^logn whose first-half descriptors start at row0 (second halves at row0 + the plan's offset).
@@ -149,7 +150,7 @@ struct hefx_bconv_plan {
     uint32_t L = 0, Lp = 0;
     std::vector<uint32_t> src, dst;
     void* d_const = nullptr;          // BConvConst (see bconv.cu)
-    void* d_bat = nullptr;            // BAT digit matrix of step 2 (fp16), see bconv.cu
+    hefx::BcTcPlan* tc = nullptr;     // tensor form, null where it does not apply
     uint32_t* d_err = nullptr;        // bounded-wait error flag of the pipelined kernels (0 = none)
 };
 
@@ -160,6 +161,8 @@ struct hefx_modup_plan {
     uint32_t L = 0, K = 0, alpha = 0, dnum = 0;
     std::vector<uint32_t> q, p;
     void* d_const = nullptr;  // dnum BConvConst
+    hefx::BcTcPlan* tc = nullptr;  // tensor form of every digit, null where it does not apply
+    uint32_t* d_err = nullptr;     // its bounded-wait error flag (0 = none)
 };
 
 namespace hefx {
@@ -245,6 +248,7 @@ cudaError_t launch_bconv_cc_tma(const hefx_bconv_plan* plan, const uint32_t* in,
                                 uint32_t* err, cudaStream_t stream);
 cudaError_t bconv_plan_upload(hefx_bconv_plan* plan);
 cudaError_t modup_plan_upload(hefx_modup_plan* plan);
+void modup_plan_free(hefx_modup_plan* plan);
 // U[b][j] = ModUp digit j of c[b] ([batch][L][N] -> [batch][dnum][L + K][N], coefficient form)
 cudaError_t launch_mod_up(const hefx_modup_plan* plan, const uint32_t* c, uint32_t* U, size_t batch,
                           cudaStream_t stream);
@@ -296,5 +300,9 @@ cudaError_t polymul_tc_noalloc(const hefx_params* p, const uint32_t* a, const ui
                                cudaStream_t stream);
 cudaError_t launch_bconv_tc(const hefx_bconv_plan* plan, const uint32_t* in, uint32_t* out, size_t batch,
                             cudaStream_t stream);
+cudaError_t launch_mod_down_tc(const hefx_bconv_plan* plan, const uint32_t* x, uint32_t* out, size_t batch,
+                               cudaStream_t stream);
+cudaError_t launch_mod_up_tc(const hefx_modup_plan* plan, const uint32_t* c, uint32_t* U, size_t batch,
+                             cudaStream_t stream);
 
 }  // namespace hefx

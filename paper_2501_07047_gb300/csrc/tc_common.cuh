@@ -55,18 +55,30 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 }
 
 // Waits for the phase with the given parity to complete; false (and *err set) once
-// `limit_ns` of %globaltimer have passed (checked every 256 polls) without it.
+// `limit_ns` of %globaltimer have passed without it, or once another thread has given up.  Both are
+// looked at every 64 polls only: a read of the flag is a trip to L2, which after each
+// failed poll would make every wait overshoot by half a trip.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint32_t* err, uint32_t code,
                                           uint64_t limit_ns = kWaitLimitNs) {
     if (mbar_try_wait(bar, parity)) return true;
     const uint64_t t0 = globaltimer();
     for (uint32_t it = 0;; ++it) {
         if (mbar_try_wait(bar, parity)) return true;
-        if ((it & 255u) == 255u && globaltimer() - t0 > limit_ns) {
+        if ((it & 63u) != 63u) continue;
+        if (*(volatile uint32_t*)err != 0u) return false;
+        if (globaltimer() - t0 > limit_ns) {
             atomicCAS(err, 0u, code);
             return false;
         }
-        if (*(volatile uint32_t*)err != 0u) return false;  // another thread already gave up
+    }
+}
+
+// Waits (bounded) for the phase whatever the error flag says: no copy may still be writing shared
+// memory when its CTA exits.
+__device__ __forceinline__ void mbar_drain(uint64_t* bar, uint32_t parity) {
+    if (mbar_try_wait(bar, parity)) return;
+    const uint64_t t0 = globaltimer();
+    while (!mbar_try_wait(bar, parity) && globaltimer() - t0 <= kWaitLimitNs) {
     }
 }
 

@@ -55,6 +55,7 @@ SIGNATURES = {
     "hefx_modup_plan_destroy": (None, [_vp]),
     "hefx_modup_plan_dnum": (_u32, [_vp]),
     "hefx_mod_up": (_i32, [_vp, _vp, _vp, _vp, _sz, _vp]),
+    "hefx_modup_check": (_i32, [_vp, _vp, _vp]),
     "hefx_rescale": (_i32, [_vp, _vp, _vp, _vp, _sz, _vp]),
     "hefx_rescale_ntt": (_i32, [_vp, _vp, _vp, _vp, _sz, _vp]),
     "hefx_ntt_inv_hadamard": (_i32, [_vp, _vp, _vp, _vp, _vp, _sz, _vp]),
@@ -276,6 +277,11 @@ def hefx_modup_plan_dnum(plan: int) -> int:
 
 def hefx_mod_up(ctx, plan, c, U, batch, stream=None) -> None:
     _check(ctx, load().hefx_mod_up(ctx, plan, _ptr(c), _ptr(U), batch, _stream(stream)))
+
+
+def hefx_modup_check(ctx, plan, stream=None) -> None:
+    """Raises HefxError(ETIMEOUT) if a bounded wait of a ModUp launched with `plan` expired."""
+    _check(ctx, load().hefx_modup_check(ctx, plan, _stream(stream)))
 
 
 def hefx_rescale(ctx, params, x, out, batch, stream=None) -> None:
