@@ -356,6 +356,25 @@ hefx_status hefx_mod_down(hefx_ctx* ctx, const hefx_bconv_plan* plan, const uint
                           size_t batch, void* stream);
 
 /*
+ * ModDown split around the inverse transform, for a result that is wanted in coefficient form
+ * (HE-Mult followed by Rescale): the inverse NTT is linear, so the scale by P^-1 and the addition
+ * of another ciphertext can be done in evaluation form where the inner product writes its limbs,
+ *   hefx_key_inner_product_add:  out[b][k][l] = (sum_j digits o evk)_l * P^-1 + add[b][k][l], l < L,
+ *                                out[b][k][l] = (sum_j digits o evk)_l                      , l >= L,
+ * and after the inverse NTT of all L + K limbs
+ *   hefx_mod_down_scaled:        out[b][j] = x[b][j] - BConv_{P->Q}(x[b][L..])_j * P^-1  mod q_j,
+ * which is ModDown(INTT(sum)) + INTT(add), with identical results.  `plan` is the conversion of
+ * hefx_mod_down (from P to Q); `params` of the inner product hold Q then P at the plan's N (EINVAL
+ * otherwise).  Layouts and errors as for hefx_key_inner_product (d_add [batch][2][L][N],
+ * evaluation form, not overlapping d_out) and hefx_mod_down.
+ */
+hefx_status hefx_key_inner_product_add(hefx_ctx* ctx, const hefx_params* params, const hefx_bconv_plan* plan,
+                                       const uint32_t* d_digits, const uint32_t* d_evk, const uint32_t* d_add,
+                                       uint32_t* d_out, uint32_t dnum, size_t batch, void* stream);
+hefx_status hefx_mod_down_scaled(hefx_ctx* ctx, const hefx_bconv_plan* plan, const uint32_t* d_x, uint32_t* d_out,
+                                 size_t batch, void* stream);
+
+/*
  * Rescale by the last prime of the parameter set (the HE operator Rescale of Sec. V-A;
  * textbook RNS-CKKS): for params over q_0..q_{L-1} (L >= 2), d_x [batch][L][N] and d_out
  * [batch][L-1][N], both in coefficient form,

@@ -144,7 +144,8 @@ constexpr int kIGroup = 8;  // source limbs whose loads are in flight together
 // MODE 4 (list): block row y converts one polynomial of an independent conversion of its own
 // (BcListEntry y: plan constants, source and output pointers; serving batches requests whose
 // source bases differ).
-enum : int { BC_FAST = 0, BC_MODDOWN = 1, BC_EXACT = 2, BC_MODUP = 3, BC_LIST = 4 };
+// MODE 5 (ModDown of scaled limbs): x_j - conv_j P^-1.
+enum : int { BC_FAST = 0, BC_MODDOWN = 1, BC_EXACT = 2, BC_MODUP = 3, BC_LIST = 4, BC_MODDOWN_SCALED = 5 };
 
 template <int kCoef>
 __host__ __device__ constexpr int log2_const() {
@@ -310,6 +311,11 @@ __global__ void __launch_bounds__(256, MODE == BC_MODUP ? 4 : 5)
                             const uint32_t xj = __ldg(xq + b * in_stride + (size_t)j * n + x0 + u * per_poly);
                             r = csub(mul_shoup_lazy(xj + pj - r, c.pinv[j], c.pinv_sh[j], pj), pj);
                         }
+                        if constexpr (MODE == BC_MODDOWN_SCALED) {
+                            const uint32_t pj = c.p[j];
+                            const uint32_t xj = __ldg(xq + b * in_stride + (size_t)j * n + x0 + u * per_poly);
+                            r = csub(xj + pj - csub(mul_shoup_lazy(r, c.pinv[j], c.pinv_sh[j], pj), pj), pj);
+                        }
                         const uint32_t jr = MODE == BC_MODUP && j >= c.skip_lo ? j + c.skip_len : j;
                         dst[(size_t)jr * n + u * per_poly] = r;
                     }
@@ -427,15 +433,21 @@ cudaError_t launch_bconv_exact(const hefx_bconv_plan* plan, const uint32_t* in, 
     return launch_cc<BC_EXACT>(plan, in, out, nullptr, batch, (size_t)plan->L << plan->log2n, stream);
 }
 
-cudaError_t launch_mod_down(const hefx_bconv_plan* plan, const uint32_t* x, uint32_t* out, size_t batch,
+const uint32_t* bconv_plan_pinv(const hefx_bconv_plan* plan) {
+    return reinterpret_cast<const uint32_t*>(static_cast<const uint8_t*>(plan->d_const) + offsetof(BConvConst, pinv));
+}
+
+cudaError_t launch_mod_down(const hefx_bconv_plan* plan, const uint32_t* x, uint32_t* out, size_t batch, bool scaled,
                             cudaStream_t stream) {
     // x: [batch][Lp + L][n] (target-basis limbs first, then the plan's source limbs)
     if (batch == 0) return cudaSuccess;
-    const cudaError_t te = launch_mod_down_tc(plan, x, out, batch, stream);
+    const cudaError_t te = launch_mod_down_tc(plan, x, out, batch, scaled, stream);
     if (te != cudaErrorNotSupported) return te;
     const size_t n = (size_t)1 << plan->log2n;
-    return launch_cc<BC_MODDOWN>(plan, x + (size_t)plan->Lp * n, out, x, batch, (size_t)(plan->L + plan->Lp) * n,
-                                 stream);
+    const size_t stride = (size_t)(plan->L + plan->Lp) * n;
+    if (scaled)
+        return launch_cc<BC_MODDOWN_SCALED>(plan, x + (size_t)plan->Lp * n, out, x, batch, stride, stream);
+    return launch_cc<BC_MODDOWN>(plan, x + (size_t)plan->Lp * n, out, x, batch, stride, stream);
 }
 
 }  // namespace hefx

@@ -5,7 +5,8 @@
 //   out_{n,j}    = ( sum_o D[n][(j, o)] 2^(8o) ) mod p_j
 //
 // b_{n,i} = [a_{n,i} qhat_i^-1]_{q_i} is step 1 (a Shoup product).  One kernel runs the plain
-// conversion, ModDown (its epilogue returns (x_j - out_j) P^-1) and ModUp (every digit in one
+// conversion, ModDown (its epilogue returns (x_j - out_j) P^-1, or x_j - out_j P^-1 where x_j carries
+// the factor already) and ModUp (every digit in one
 // launch).
 //
 // What bounds it: memory, once the work per (coefficient, limb) is small enough.  The MMAs are
@@ -83,7 +84,9 @@ struct BcTcConst {
 static_assert(sizeof(BcTcConst) % 16 == 0, "copied as uint4");
 
 // BT_SMALL: the plain conversion with a target below 2^18.
-enum : int { BT_FAST = 0, BT_MODDOWN = 1, BT_MODUP = 2, BT_SMALL = 3 };
+enum : int { BT_FAST = 0, BT_MODDOWN = 1, BT_MODUP = 2, BT_SMALL = 3, BT_MODDOWN_SCALED = 4 };
+template <int MODE>
+constexpr bool kModDown = MODE == BT_MODDOWN || MODE == BT_MODDOWN_SCALED;
 
 // Shared-memory layout of a launch, sized for its largest conversion (bytes from a 1 KiB-aligned base).
 struct BcTcLayout {
@@ -413,7 +416,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             const size_t x = (size_t)(t & ((1u << logt) - 1)) * TILE + row;
             char* dst = reinterpret_cast<char*>(out + (size_t)(t >> logt) * a.out_stride + x);
             [[maybe_unused]] const char* xq = nullptr;
-            if constexpr (MODE == BT_MODDOWN)
+            if constexpr (kModDown<MODE>)
                 xq = reinterpret_cast<const char*>(a.xq + (size_t)(t >> logt) * a.xq_stride + x);
             // eight targets (two 16-column reads) at a time
             auto group8 = [&](uint32_t j0, auto full) {
@@ -422,7 +425,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                 if (decltype(full)::value || j0 + 4 < Lp)
                     tc::tmem_ld16(cols + j0 * 4 + 16, *reinterpret_cast<uint32_t(*)[16]>(&r[16]));
                 [[maybe_unused]] uint32_t xv[8];
-                if constexpr (MODE == BT_MODDOWN) {
+                if constexpr (kModDown<MODE>) {
 #pragma unroll
                     for (uint32_t h = 0; h < 8; ++h)
                         xv[h] = decltype(full)::value || j0 + h < Lp
@@ -441,9 +444,12 @@ __global__ void __launch_bounds__(THREADS, 1)
                     } else {
                         v[h] = barrett64((uint64_t)lo + ((uint64_t)(hr - 0x43000000u) << 16), q.x, c.mu64[j0 + h]);
                     }
-                    if constexpr (MODE == BT_MODDOWN) {
+                    if constexpr (kModDown<MODE>) {
                         const uint2 w = *(reinterpret_cast<const uint2*>(&c.tgt[j0 + h]) + 1);
-                        v[h] = csub(mul_shoup_lazy(xv[h] + q.x - v[h], w.x, w.y, q.x), q.x);
+                        if constexpr (MODE == BT_MODDOWN)
+                            v[h] = csub(mul_shoup_lazy(xv[h] + q.x - v[h], w.x, w.y, q.x), q.x);
+                        else
+                            v[h] = csub(xv[h] + q.x - csub(mul_shoup_lazy(v[h], w.x, w.y, q.x), q.x), q.x);
                     }
                 }
 #pragma unroll
@@ -678,7 +684,7 @@ cudaError_t launch_bconv_tc(const hefx_bconv_plan* plan, const uint32_t* in, uin
 }
 
 cudaError_t launch_mod_down_tc(const hefx_bconv_plan* plan, const uint32_t* x, uint32_t* out, size_t batch,
-                               cudaStream_t stream) {
+                               bool scaled, cudaStream_t stream) {
     if (!bconv_prefer_tc(plan, batch) || plan->tc->small_target) return cudaErrorNotSupported;
     BcTcArgs a = {};
     a.out = out;
@@ -686,6 +692,9 @@ cudaError_t launch_mod_down_tc(const hefx_bconv_plan* plan, const uint32_t* x, u
     a.xq_stride = (size_t)(plan->L + plan->Lp) << plan->log2n;
     a.out_stride = (size_t)plan->Lp << plan->log2n;
     a.err = plan->d_err;
+    if (scaled)
+        return launch_plan<BT_MODDOWN_SCALED>(plan->tc, a, x, plan->L + plan->Lp, plan->Lp, plan->log2n, batch,
+                                              (size_t)sm_count(), 1, stream);
     return launch_plan<BT_MODDOWN>(plan->tc, a, x, plan->L + plan->Lp, plan->Lp, plan->log2n, batch,
                                    (size_t)sm_count(), 1, stream);
 }

@@ -96,9 +96,15 @@ __device__ __forceinline__ uint32_t kip_final(uint32_t acc, const LimbConst& c) 
     return csub(mul_mont_lazy(acc, c.r2, c.q, c.qinv_neg), c.q);
 }
 
+// ADD: the limbs of Q (the first lq) return sum * P^-1 + add[b][k][l] instead of the sum, with pinv[l] =
+// P^-1 mod q_l: the ModDown scale and the ciphertext addition, which a later pass would read and
+// write every limb for (memory binds: 256 MB at (48, 28, 3) take 38 us, 36 without the addend).
+template <bool ADD>
 __global__ void __launch_bounds__(256) key_inner_product_kernel(const LimbConst* __restrict__ lc, uint32_t nl,
                                                                 uint32_t n, uint32_t dnum, size_t batch,
-                                                                const uint4* dig, const uint4* evk, uint4* out) {
+                                                                const uint4* dig, const uint4* evk, uint4* out,
+                                                                uint32_t lq, const uint32_t* __restrict__ pinv,
+                                                                const uint4* add) {
     griddep_wait();
     const size_t per_poly4 = (size_t)nl * n / 4;  // uint4 groups of one polynomial over Q u P
     const size_t total4 = batch * per_poly4;
@@ -114,10 +120,24 @@ __global__ void __launch_bounds__(256) key_inner_product_kernel(const LimbConst*
             a1 = make_uint4(kip_term(a1.x, d.x, k1.x, c), kip_term(a1.y, d.y, k1.y, c), kip_term(a1.z, d.z, k1.z, c),
                             kip_term(a1.w, d.w, k1.w, c));
         }
-        out[(2 * b) * per_poly4 + e] = make_uint4(kip_final(a0.x, c), kip_final(a0.y, c), kip_final(a0.z, c),
-                                                  kip_final(a0.w, c));
-        out[(2 * b + 1) * per_poly4 + e] = make_uint4(kip_final(a1.x, c), kip_final(a1.y, c), kip_final(a1.z, c),
-                                                      kip_final(a1.w, c));
+        uint4 r0, r1;
+        if (ADD && (e * 4) / n < lq) {
+            // P^-1 2^64 mod q: the Montgomery factor of the sum (2^64, r2) and the scale in one
+            const uint32_t p32 = csub(mul_mont_lazy(c.r2, __ldg(pinv + (e * 4) / n), c.q, c.qinv_neg), c.q);
+            const uint32_t s = csub(mul_mont_lazy(p32, c.r2, c.q, c.qinv_neg), c.q);
+            const size_t q4 = (size_t)lq * n / 4;
+            const uint4 d0 = add[(2 * b) * q4 + e], d1 = add[(2 * b + 1) * q4 + e];
+            auto one = [&](uint32_t acc, uint32_t d) {
+                return csub(csub(mul_mont_lazy(acc, s, c.q, c.qinv_neg), c.q) + d, c.q);
+            };
+            r0 = make_uint4(one(a0.x, d0.x), one(a0.y, d0.y), one(a0.z, d0.z), one(a0.w, d0.w));
+            r1 = make_uint4(one(a1.x, d1.x), one(a1.y, d1.y), one(a1.z, d1.z), one(a1.w, d1.w));
+        } else {
+            r0 = make_uint4(kip_final(a0.x, c), kip_final(a0.y, c), kip_final(a0.z, c), kip_final(a0.w, c));
+            r1 = make_uint4(kip_final(a1.x, c), kip_final(a1.y, c), kip_final(a1.z, c), kip_final(a1.w, c));
+        }
+        out[(2 * b) * per_poly4 + e] = r0;
+        out[(2 * b + 1) * per_poly4 + e] = r1;
     }
 }
 
@@ -199,8 +219,19 @@ cudaError_t launch_key_inner_product(const hefx_params* p, const uint32_t* dig, 
                                      uint32_t dnum, size_t batch, cudaStream_t s) {
     const size_t total4 = batch * p->nlimbs * p->n / 4;
     if (!total4) return cudaSuccess;
-    return launch_pdl(key_inner_product_kernel, grid_for(total4), 256, 0, s, (const LimbConst*)p->d_lc, p->nlimbs, p->n,
-                      dnum, batch, (const uint4*)dig, (const uint4*)evk, (uint4*)out);
+    return launch_pdl(key_inner_product_kernel<false>, grid_for(total4), 256, 0, s, (const LimbConst*)p->d_lc,
+                      p->nlimbs, p->n, dnum, batch, (const uint4*)dig, (const uint4*)evk, (uint4*)out, 0u,
+                      (const uint32_t*)nullptr, (const uint4*)nullptr);
+}
+
+cudaError_t launch_key_inner_product_add(const hefx_params* p, const uint32_t* dig, const uint32_t* evk,
+                                         const uint32_t* add, uint32_t lq, const uint32_t* d_pinv, uint32_t* out,
+                                         uint32_t dnum, size_t batch, cudaStream_t s) {
+    const size_t total4 = batch * p->nlimbs * p->n / 4;
+    if (!total4) return cudaSuccess;
+    return launch_pdl(key_inner_product_kernel<true>, grid_for(total4), 256, 0, s, (const LimbConst*)p->d_lc,
+                      p->nlimbs, p->n, dnum, batch, (const uint4*)dig, (const uint4*)evk, (uint4*)out, lq, d_pinv,
+                      (const uint4*)add);
 }
 
 cudaError_t launch_rescale(const hefx_params* p, const uint32_t* x, uint32_t* out, size_t batch, cudaStream_t s) {

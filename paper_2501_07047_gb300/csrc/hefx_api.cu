@@ -675,6 +675,32 @@ hefx_status hefx_key_inner_product(hefx_ctx* ctx, const hefx_params* p, const ui
     return HEFX_OK;
 }
 
+hefx_status hefx_key_inner_product_add(hefx_ctx* ctx, const hefx_params* p, const hefx_bconv_plan* plan,
+                                       const uint32_t* digits, const uint32_t* evk, const uint32_t* add, uint32_t* out,
+                                       uint32_t dnum, size_t batch, void* stream) {
+    hefx_status st;
+    if ((st = check_ntt_args(ctx, p, digits, "d_digits")) != HEFX_OK) return st;
+    if ((st = check_ntt_args(ctx, p, evk, "d_evk")) != HEFX_OK) return st;
+    if ((st = check_ntt_args(ctx, p, add, "d_add")) != HEFX_OK) return st;
+    if ((st = check_ntt_args(ctx, p, out, "d_out")) != HEFX_OK) return st;
+    if (!plan || plan->ctx != ctx) return fail(ctx, HEFX_EINVAL, "plan is null or belongs to another context");
+    if (dnum == 0 || dnum > 64) return fail(ctx, HEFX_EINVAL, "dnum = %u outside [1, 64]", dnum);
+    bool match = plan->log2n == p->log2n && plan->L + plan->Lp == p->nlimbs;
+    for (uint32_t l = 0; match && l < p->nlimbs; ++l)
+        match = p->primes[l] == (l < plan->Lp ? plan->dst[l] : plan->src[l - plan->Lp]);
+    if (!match) return fail(ctx, HEFX_EINVAL, "params must hold the plan's targets, then its sources, at its N");
+    const size_t poly = (size_t)p->nlimbs * p->n * 4, qpoly = (size_t)plan->Lp * p->n * 4;
+    if (overlaps(out, batch * 2 * poly, digits, batch * dnum * poly) || overlaps(out, batch * 2 * poly, evk, dnum * 2 * poly) ||
+        overlaps(out, batch * 2 * poly, add, batch * 2 * qpoly))
+        return fail(ctx, HEFX_EINVAL, "d_out overlaps an input");
+    if (batch == 0) return HEFX_OK;
+    if ((st = use_device(ctx)) != HEFX_OK) return st;
+    cudaError_t e = launch_key_inner_product_add(p, digits, evk, add, plan->Lp, bconv_plan_pinv(plan), out, dnum, batch,
+                                                 (cudaStream_t)stream);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "hefx_key_inner_product_add launch");
+    return HEFX_OK;
+}
+
 hefx_status hefx_rescale(hefx_ctx* ctx, const hefx_params* p, const uint32_t* x, uint32_t* out, size_t batch,
                          void* stream) {
     hefx_status st;
@@ -710,8 +736,8 @@ hefx_status hefx_rescale_ntt(hefx_ctx* ctx, const hefx_params* p, const uint32_t
     return HEFX_OK;
 }
 
-hefx_status hefx_mod_down(hefx_ctx* ctx, const hefx_bconv_plan* plan, const uint32_t* x, uint32_t* out, size_t batch,
-                          void* stream) {
+static hefx_status mod_down(hefx_ctx* ctx, const hefx_bconv_plan* plan, const uint32_t* x, uint32_t* out, size_t batch,
+                            bool scaled, void* stream, const char* name) {
     if (!ctx) return HEFX_EINVAL;
     if (!plan || plan->ctx != ctx) return fail(ctx, HEFX_EINVAL, "plan is null or belongs to another context");
     if (!x || !out) return fail(ctx, HEFX_EINVAL, "null buffer");
@@ -722,9 +748,19 @@ hefx_status hefx_mod_down(hefx_ctx* ctx, const hefx_bconv_plan* plan, const uint
     hefx_status st = use_device(ctx);
     if (st != HEFX_OK) return st;
     if (batch == 0) return HEFX_OK;
-    cudaError_t e = launch_mod_down(plan, x, out, batch, (cudaStream_t)stream);
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "hefx_mod_down launch");
+    cudaError_t e = launch_mod_down(plan, x, out, batch, scaled, (cudaStream_t)stream);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, name);
     return HEFX_OK;
+}
+
+hefx_status hefx_mod_down(hefx_ctx* ctx, const hefx_bconv_plan* plan, const uint32_t* x, uint32_t* out, size_t batch,
+                          void* stream) {
+    return mod_down(ctx, plan, x, out, batch, false, stream, "hefx_mod_down launch");
+}
+
+hefx_status hefx_mod_down_scaled(hefx_ctx* ctx, const hefx_bconv_plan* plan, const uint32_t* x, uint32_t* out,
+                                 size_t batch, void* stream) {
+    return mod_down(ctx, plan, x, out, batch, true, stream, "hefx_mod_down_scaled launch");
 }
 
 hefx_status hefx_tensor_product(hefx_ctx* ctx, const hefx_params* p, const uint32_t* a0, const uint32_t* a1,

@@ -235,11 +235,17 @@ cudaError_t launch_vec_mod_add(const hefx_params* p, const uint32_t* x, const ui
                                cudaStream_t s);
 cudaError_t launch_key_inner_product(const hefx_params* p, const uint32_t* dig, const uint32_t* evk, uint32_t* out,
                                      uint32_t dnum, size_t batch, cudaStream_t s);
+// The inner product with the ModDown scale and an addend on the first lq limbs (d_pinv: P^-1 mod q_l).
+cudaError_t launch_key_inner_product_add(const hefx_params* p, const uint32_t* dig, const uint32_t* evk,
+                                         const uint32_t* add, uint32_t lq, const uint32_t* d_pinv, uint32_t* out,
+                                         uint32_t dnum, size_t batch, cudaStream_t s);
 cudaError_t launch_rescale(const hefx_params* p, const uint32_t* x, uint32_t* out, size_t batch, cudaStream_t s);
 cudaError_t launch_bconv_exact(const hefx_bconv_plan* plan, const uint32_t* in, uint32_t* out, size_t batch,
                                cudaStream_t stream);
-cudaError_t launch_mod_down(const hefx_bconv_plan* plan, const uint32_t* x, uint32_t* out, size_t batch,
+// scaled: x's ciphertext limbs already carry the factor P^-1 (only the conversion is multiplied by it)
+cudaError_t launch_mod_down(const hefx_bconv_plan* plan, const uint32_t* x, uint32_t* out, size_t batch, bool scaled,
                             cudaStream_t stream);
+const uint32_t* bconv_plan_pinv(const hefx_bconv_plan* plan);  // device: (prod q_i)^-1 mod p_j
 cudaError_t launch_bconv_cc(const hefx_bconv_plan* plan, const uint32_t* in, uint32_t* out, size_t batch,
                             cudaStream_t stream);
 // The plain conversion with TMA-fed tiles (bconv_cc_tma.cu): L <= 48 sources, N >= 2^8;
@@ -301,7 +307,7 @@ cudaError_t polymul_tc_noalloc(const hefx_params* p, const uint32_t* a, const ui
 cudaError_t launch_bconv_tc(const hefx_bconv_plan* plan, const uint32_t* in, uint32_t* out, size_t batch,
                             cudaStream_t stream);
 cudaError_t launch_mod_down_tc(const hefx_bconv_plan* plan, const uint32_t* x, uint32_t* out, size_t batch,
-                               cudaStream_t stream);
+                               bool scaled, cudaStream_t stream);
 cudaError_t launch_mod_up_tc(const hefx_modup_plan* plan, const uint32_t* c, uint32_t* U, size_t batch,
                              cudaStream_t stream);
 

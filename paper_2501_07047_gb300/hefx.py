@@ -51,6 +51,8 @@ SIGNATURES = {
     "hefx_bconv_check": (_i32, [_vp, _vp, _vp]),
     "hefx_key_inner_product": (_i32, [_vp, _vp, _vp, _vp, _vp, _u32, _sz, _vp]),
     "hefx_mod_down": (_i32, [_vp, _vp, _vp, _vp, _sz, _vp]),
+    "hefx_mod_down_scaled": (_i32, [_vp, _vp, _vp, _vp, _sz, _vp]),
+    "hefx_key_inner_product_add": (_i32, [_vp, _vp, _vp, _vp, _vp, _vp, _vp, _u32, _sz, _vp]),
     "hefx_modup_plan_create": (_i32, [_vp, _u32, _u32p, _u32, _u32p, _u32, _u32, ctypes.POINTER(_vp)]),
     "hefx_modup_plan_destroy": (None, [_vp]),
     "hefx_modup_plan_dnum": (_u32, [_vp]),
@@ -258,6 +260,15 @@ def hefx_basis_convert_exact(ctx, plan, x, out, batch, stream=None) -> None:
 
 def hefx_mod_down(ctx, plan, x, out, batch, stream=None) -> None:
     _check(ctx, load().hefx_mod_down(ctx, plan, _ptr(x), _ptr(out), batch, _stream(stream)))
+
+
+def hefx_mod_down_scaled(ctx, plan, x, out, batch, stream=None) -> None:
+    _check(ctx, load().hefx_mod_down_scaled(ctx, plan, _ptr(x), _ptr(out), batch, _stream(stream)))
+
+
+def hefx_key_inner_product_add(ctx, params, plan, digits, evk, add, out, dnum, batch, stream=None) -> None:
+    _check(ctx, load().hefx_key_inner_product_add(ctx, params, plan, _ptr(digits), _ptr(evk), _ptr(add), _ptr(out),
+                                                  dnum, batch, _stream(stream)))
 
 
 def hefx_modup_plan_create(ctx: int, log2n: int, q, p, alpha: int) -> int:

@@ -12,6 +12,11 @@ and VecModAdd (App. A); it does not print their formulas, which here are textboo
   ks_k = ModDown(INTT(acc_k)), c_k = d_k + NTT(ks_k)
   c'_k = NTT(Rescale(INTT(c_k)))                          over q_0 .. q_{L-2}
 
+With the Rescale, INTT(c_k) = INTT(d_k) + ks_k is all that is needed of c_k, and by linearity it is
+t_k - P^-1 BConv_{P->Q}(INTT(acc_k)_P) with t_k = INTT(P^-1 acc_k + d_k) over Q: the key inner product
+scales and adds as it writes, and two transforms of c (NTT(ks), INTT(c), 96 limbs each at L = 48)
+and the addition drop out.
+
 Every step runs in libhefx's kernels; this module only allocates workspaces and issues the
 calls on one stream.  Inputs and outputs are one ciphertext pair in evaluation form.
 """
@@ -63,6 +68,7 @@ class HeMult:
         self.acc = torch.empty((2, L + K, n), dtype=torch.int32, device=dev)
         self.ks = torch.empty((2, L, n), dtype=torch.int32, device=dev)
         self.cc = torch.empty((2, L, n), dtype=torch.int32, device=dev)
+        self.merged = False  # the last run took the merged form (stages)
 
     def close(self) -> None:
         if self.modup:
@@ -78,7 +84,7 @@ class HeMult:
     def launches(self, rescale: bool = True) -> int:
         """Kernel launches of one run (CUDA-core NTT path)."""
         modup = 1 if self.modup else sum(2 if lo else 1 for lo, _ in self.digits)
-        return 1 + 1 + modup + 1 + 1 + 1 + 1 + 1 + 1 + (2 if rescale else 0)
+        return 1 + 1 + modup + 1 + 1 + 1 + 1 + (1 if rescale else 2)
 
     def run(self, a0, a1, b0, b1, evk, out, stream=None, rescale: bool = True) -> None:
         """a*, b*: [L][N] evaluation form over Q; evk: [dnum][2][L+K][N] evaluation form over
@@ -107,6 +113,14 @@ class HeMult:
                     hefx.hefx_basis_convert(ctx, lo_plan, self.c[lo:hi], self.U[j, :lo], 1, self.bconv_path, st)
                 hefx.hefx_basis_convert(ctx, hi_plan, self.c[lo:hi], self.U[j, hi:], 1, self.bconv_path, st)
             hefx.hefx_ntt_fwd(ctx, self.pQP, self.U, self.dnum, self.ntt_path, st)
+            self.merged = rescale and self.ntt_path == "cudacore"
+            if self.merged:
+                hefx.hefx_key_inner_product_add(ctx, self.pQP, self.plan_pq, self.U, evk, self.d[0:2], self.acc,
+                                                self.dnum, 1, st)
+                hefx.hefx_ntt_inv(ctx, self.pQP, self.acc, 2, self.ntt_path, st)
+                hefx.hefx_mod_down_scaled(ctx, self.plan_pq, self.acc, self.cc, 2, st)
+                hefx.hefx_rescale_ntt(ctx, self.pQ, self.cc, out, 2, st)
+                return
             hefx.hefx_key_inner_product(ctx, self.pQP, self.U, evk, self.acc, self.dnum, 1, st)
             hefx.hefx_ntt_inv(ctx, self.pQP, self.acc, 2, self.ntt_path, st)
             hefx.hefx_mod_down(ctx, self.plan_pq, self.acc, self.ks, 2, st)
@@ -148,6 +162,23 @@ class HeMult:
         return g
 
     def stages(self) -> dict:
-        """The workspaces after a run (for stage-by-stage parity tests)."""
-        return {"d0": self.d[0], "d1": self.d[1], "d2_coeff": self.c, "modup_eval": self.U, "acc_coeff": self.acc,
-                "ks_eval": self.ks, "c_coeff": self.cc}
+        """The workspaces after a run (for stage-by-stage parity tests).  The merged form keeps
+        t (P^-1 acc + d over Q, acc over P) and c in coefficient form; the stages that it does not
+        compute are worked out from those here."""
+        torch = self.torch
+        st = {"d0": self.d[0], "d1": self.d[1], "d2_coeff": self.c, "modup_eval": self.U, "c_coeff": self.cc}
+        if not self.merged:
+            return {**st, "acc_coeff": self.acc, "ks_eval": self.ks}
+        s = torch.cuda.current_stream()
+        q = torch.tensor(self.qs, dtype=torch.int64, device="cuda")[None, :, None]
+        P = 1
+        for p in self.ps:
+            P *= p
+        pmod = torch.tensor([P % v for v in self.qs], dtype=torch.int64, device="cuda")[None, :, None]
+        d = self.d[0:2].clone()
+        hefx.hefx_ntt_inv(self.ctx, self.pQ, d, 2, self.ntt_path, s)
+        acc = self.acc.clone()
+        acc[:, :self.L] = ((self.acc[:, :self.L].long() - d.long() + q) * pmod % q).to(torch.int32)
+        ks = ((self.cc.long() - d.long() + q) % q).to(torch.int32)
+        hefx.hefx_ntt_fwd(self.ctx, self.pQ, ks, 2, self.ntt_path, s)
+        return {**st, "acc_coeff": acc, "ks_eval": ks}
