@@ -276,18 +276,17 @@ def run_gpu(args):
         st = hefx.raw_status("hefx_ntt_fwd", ctx, params, data.data_ptr(), 0, hefx.PATHS[path], stream.cuda_stream)
         return st == hefx.HEFX_OK
 
-    # timed configurations: the CUDA-core path under both of its schedules (one launch of 8-CTA
-    # clusters; two launches, column pass then block pass) and the tensor path with each split
-    # and GEMM tile width
-    configs = [("cudacore", "cudacore", 0, (0, 0), "auto"), ("cudacore_2p", "cudacore", 0, (0, 0), "two_pass")]
+    # timed configurations: the CUDA-core path under both of its schedules (the library's choice,
+    # which is two launches, strided pass and block pass, at 192 rows; one launch of 8-CTA
+    # clusters) and the tensor path with each split and GEMM tile width
+    configs = [("cudacore", "cudacore", 0, (0, 0), "auto"), ("cudacore_cluster", "cudacore", 0, (0, 0), "cluster")]
     if available("tensor"):
         # two-factor 256 x 256 and the three-factor 64 x 32 x 32 split, each with both tiles
         configs += [("tensor", "tensor", 64, (0, 0), "auto"), ("tensor_t32", "tensor", 32, (0, 0), "auto"),
                     ("tensor_3f", "tensor", 64, (6, 5), "auto"), ("tensor_3f_t32", "tensor", 32, (6, 5), "auto")]
     # Whole-job throughput: the K steps are independent batches, and a stream of them runs
     # with steps k and k + 1 overlapping on PIPE_STREAMS streams, so that the GPU is not idle
-    # in each transform's last, partial wave of clusters (192 rows over 89 co-resident
-    # clusters leave about a fifth of a launch nearly empty).  PIPE_BATCHES rotating input
+    # in each launch's last, partial wave of CTAs.  PIPE_BATCHES rotating input
     # batches of 48 MiB (192 MiB) exceed L2, so these steps need no flush.  One parameter set
     # per stream: the tensor path's digit workspace lives in the parameter set.  The
     # per-launch times (fwd_ms / inv_ms, the roofline) come from the serialized loop below.
@@ -385,7 +384,7 @@ def run_gpu(args):
             "value": job_value(world, UNITS_PER_STEP, args.steps, total_ms),
             "fwd_ms": statistics.mean(fwd_ms), "inv_ms": statistics.mean(inv_ms),
             "wall_s": t_wall, "clocks": clk.summary(),
-            "launches_per_step": (4 if sched == "two_pass" else 2) if path == "cudacore" else (6 if not split[1] else 8),
+            "launches_per_step": (2 if sched == "cluster" else 4) if path == "cudacore" else (6 if not split[1] else 8),
         }
         pipe_ms, pipe_clk = pipelined(path, tile, split, sched)
         results[name].update({"ms_per_step_pipelined": pipe_ms / args.steps,
@@ -394,9 +393,9 @@ def run_gpu(args):
 
     if available("tensor"):
         hefx.hefx_params_set_tensor_config(ctx, params, 0, 64, 0)
-    # the headline is the library's own choice for this shape (AUTO: the cluster schedule at 192
-    # rows) or a tensor configuration; the explicit two-pass schedule is listed for comparison
-    best_name = max((k for k in results if k != "cudacore_2p"), key=lambda p: results[p]["value_pipelined"])
+    # the headline is the library's own choice for this shape (AUTO: the two-pass schedule at 192
+    # rows) or a tensor configuration; the explicit cluster schedule is listed for comparison
+    best_name = max((k for k in results if k != "cudacore_cluster"), key=lambda p: results[p]["value_pipelined"])
     r = results[best_name]
     best = r["path"]
     hefx.hefx_params_set_cc_schedule(ctx, params, r["schedule"])
@@ -435,11 +434,11 @@ def run_gpu(args):
         dom = max(rr["fwd_ms"], rr["inv_ms"])
         achieved = units_per_launch * BYTES_PER_UNIT / (dom / 1e3) / 1e9
         which = "fwd" if rr["fwd_ms"] >= rr["inv_ms"] else "inv"
-        cluster = rr["schedule"] != "two_pass"  # AUTO runs the cluster kernel at 192 rows
+        cluster = rr["schedule"] == "cluster"  # AUTO runs the two-pass kernels at 192 rows
         return {"bound": "hbm", "achieved": round(achieved, 1), "peak": hbm, "unit": "GB/s",
-                "frac": round(achieved / hbm, 4), "traffic": profile_traffic("ntt_cc", which) if cluster else None,
+                "frac": round(achieved / hbm, 4), "traffic": profile_traffic("ntt_cc" if cluster else "ntt_cc_2p", which),
                 "kernel": ("ntt_cc_kernel<16, " + which.upper() + ">") if cluster else
-                          ("two-pass " + which + " transform (column and block kernels, timed together)"),
+                          ("two-pass " + which + " transform (cc2::strided_kernel and block_kernel, timed together)"),
                 "algorithmic_bytes_per_launch": units_per_launch * BYTES_PER_UNIT,
                 "peak_source": f"{src} hbm_gbs"}
 

@@ -163,16 +163,14 @@ hefx_status hefx_params_set_reduction(hefx_params* params, hefx_reduction ntt_re
  *    its three cross-CTA stages go through distributed shared memory.
  *  - HEFX_CC_TWO_PASS (N = 2^16 only): two launches through L2, the row / column
  *    factorisation of the matrix NTT (Sec. IV-B) with the twiddle step folded into the
- *    butterflies: 8 stages within columns j mod 256, then 8 within 256-element blocks
- *    (reversed for the inverse); the intermediate goes through the output buffer.
- *  - HEFX_CC_AUTO (default): at N = 2^16, HEFX_CC_TWO_PASS for at most 32 rows (so few
- *    clusters leave most of the GPU idle; measured 20 % faster for one polynomial of 24
- *    limbs) and for one to one and a half waves of co-resident clusters (the cluster
- *    kernel's second wave mostly empty; 4-14 % faster at 96 and 120 rows), else
+ *    butterflies: log2 N - 10 stages over elements 1024 apart, then 10 within 1024-element
+ *    blocks (reversed for the inverse); the intermediate goes through the output buffer.
+ *  - HEFX_CC_AUTO (default): at N = 2^14 .. 2^17 the two-pass form while the intermediate stays
+ *    in L2 (forward up to 256 rows of 2^16 elements, inverse 320, rescaling forward 144), and at
+ *    N = 2^17, for the inverse at N = 2^16 and for that of a Hadamard product always; else
  *    HEFX_CC_CLUSTER.
- * Hadamard-fused forms (hefx_poly_mul), Rescale, row lists and batch plans use the cluster
- * schedule.  Errors: EINVAL (unknown schedule), EUNSUPPORTED (HEFX_CC_TWO_PASS at
- * N != 2^16).  Not thread-safe with concurrent calls that use the same params.
+ * The second half of hefx_poly_mul and fused batch plans use the cluster schedule.  Errors:
+ * EINVAL (unknown schedule), EUNSUPPORTED (HEFX_CC_TWO_PASS at N != 2^16).  Not thread-safe with concurrent calls that use the same params.
  */
 typedef enum { HEFX_CC_AUTO = 0, HEFX_CC_CLUSTER = 1, HEFX_CC_TWO_PASS = 2 } hefx_cc_schedule;
 hefx_status hefx_params_set_cc_schedule(hefx_params* params, hefx_cc_schedule schedule);

@@ -250,8 +250,6 @@ hefx_status hefx_params_create(hefx_ctx* ctx, uint32_t log2n, const uint32_t* pr
     for (uint32_t i = 0; i < nlimbs; ++i) p->max_prime = std::max(p->max_prime, primes[i]);
     std::vector<LimbConst> lc(nlimbs);
     std::vector<uint2> twf((size_t)nlimbs * n), twi((size_t)nlimbs * n);
-    const bool two_pass = log2n == 16;
-    std::vector<uint2> twf2(two_pass ? twf.size() : 0), twi2(two_pass ? twi.size() : 0);
     std::vector<uint64_t> pw(n), pwi(n);
     for (uint32_t l = 0; l < nlimbs; ++l) {
         const uint64_t q = primes[l];
@@ -267,8 +265,6 @@ hefx_status hefx_params_create(hefx_ctx* ctx, uint32_t log2n, const uint32_t* pr
         // G = J 2^v + g of sub-transform J sits at stage_base + g * (N / 2^RS) + J, so the
         // lanes of a warp (consecutive J) read consecutive entries (MAT's offline
         // reordering of constants, Sec. IV-B, applied to the table layout).
-        // The two-pass transform at N = 2^16 (ntt_cc_2p.cu) reads a second copy whose
-        // group-major part covers its 4-stage smallest-stride pass.
         auto fwd_pos = [&](uint64_t k, int RS) -> uint64_t {
             if (k == 0) return 0;
             int s = 63 - __builtin_clzll(k);  // stage of entry k: k in [2^s, 2^(s+1))
@@ -293,10 +289,6 @@ hefx_status hefx_params_create(hefx_ctx* ctx, uint32_t log2n, const uint32_t* pr
             const uint2 wi = make_uint2((uint32_t)pwi[r], shoup(pwi[r], q));
             twf[l * n + fwd_pos(k, RS)] = wf;
             twi[l * n + inv_pos(k, RS)] = wi;
-            if (two_pass) {
-                twf2[l * n + fwd_pos(k, 4)] = wf;
-                twi2[l * n + inv_pos(k, 4)] = wi;
-            }
         }
         LimbConst& c = lc[l];
         memset(&c, 0, sizeof c);
@@ -337,14 +329,6 @@ hefx_status hefx_params_create(hefx_ctx* ctx, uint32_t log2n, const uint32_t* pr
     if (e == cudaSuccess) e = cudaMemcpy(p->d_lc, lc.data(), sizeof(LimbConst) * nlimbs, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(p->d_tw_fwd, twf.data(), sizeof(uint2) * twf.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(p->d_tw_inv, twi.data(), sizeof(uint2) * twi.size(), cudaMemcpyHostToDevice);
-    if (two_pass) {
-        if (e == cudaSuccess) e = cudaMalloc(&p->d_tw2_fwd, sizeof(uint2) * twf2.size());
-        if (e == cudaSuccess) e = cudaMalloc(&p->d_tw2_inv, sizeof(uint2) * twi2.size());
-        if (e == cudaSuccess)
-            e = cudaMemcpy(p->d_tw2_fwd, twf2.data(), sizeof(uint2) * twf2.size(), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess)
-            e = cudaMemcpy(p->d_tw2_inv, twi2.data(), sizeof(uint2) * twi2.size(), cudaMemcpyHostToDevice);
-    }
     if (e != cudaSuccess) {
         hefx_params_destroy(p);
         return cuda_fail(ctx, e, "parameter tables");
@@ -363,8 +347,6 @@ void hefx_params_destroy(hefx_params* p) {
     if (p->d_lc) cudaFree(p->d_lc);
     if (p->d_tw_fwd) cudaFree(p->d_tw_fwd);
     if (p->d_tw_inv) cudaFree(p->d_tw_inv);
-    if (p->d_tw2_fwd) cudaFree(p->d_tw2_fwd);
-    if (p->d_tw2_inv) cudaFree(p->d_tw2_inv);
     if (p->d_err_cc) cudaFree(p->d_err_cc);
     if (p->d_tw_fwd_mont) cudaFree(p->d_tw_fwd_mont);
     if (p->d_tw_inv_mont) cudaFree(p->d_tw_inv_mont);
@@ -1097,7 +1079,7 @@ hefx_status hefx_params_set_cc_schedule(hefx_params* p, hefx_cc_schedule schedul
     if (!p) return HEFX_EINVAL;
     if (schedule != HEFX_CC_AUTO && schedule != HEFX_CC_CLUSTER && schedule != HEFX_CC_TWO_PASS)
         return fail(p->ctx, HEFX_EINVAL, "unknown CUDA-core schedule %d", (int)schedule);
-    if (schedule == HEFX_CC_TWO_PASS && !p->d_tw2_fwd)
+    if (schedule == HEFX_CC_TWO_PASS && p->log2n != 16)
         return fail(p->ctx, HEFX_EUNSUPPORTED, "the two-pass schedule is built for N = 2^16 only");
     p->cc_schedule = (int)schedule;
     return HEFX_OK;

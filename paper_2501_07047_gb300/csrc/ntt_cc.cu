@@ -2,6 +2,7 @@
 // instantiated per ring-degree range in ntt_cc_range_*.cu (parallel compilation).
 #include <cstring>
 
+#include "ntt_cc_2p.cuh"
 #include "ntt_cc_impl.cuh"
 
 namespace hefx {
@@ -10,12 +11,35 @@ cudaError_t launch_dispatch(const hefx_params* p, NttMode mode, const cc::KArgs&
 
 namespace {
 
-// Co-resident clusters of the N = 2^16 forward / inverse kernel, queried once per context.
-int clusters16(hefx_ctx* c, NttMode mode, bool lazy) {
-    std::lock_guard<std::mutex> g(c->mu);
-    int& v = c->cc16_clusters[mode == MODE_INV ? 1 : 0][lazy ? 1 : 0];
-    if (v < 0) v = cc::max_clusters_16(mode, lazy);
-    return v;
+// The two-pass schedule (ntt_cc_2p.cuh) is built for N = 2^14 .. 2^17 and every mode but the product's
+// second half, which would need a workspace for NTT(b).  AUTO takes it always at N = 2^17 and for the
+// inverse of a Hadamard product; else while the rows' elements are at most: forward 256 x 2^16,
+// inverse 320 x 2^16 (at N = 2^16 always), rescaling forward 144 x 2^16.  Beyond, the
+// intermediate leaves L2 between the launches and the cluster kernel's single trip through HBM
+// wins (us, cluster / two-pass):
+//   N = 2^16   24 rows     96          144         240         288         384
+//   forward    10.1 / 8.5  27.0 / 22.8 33.1 / 31.0 50.2 / 48.8 59.2 / 59.3 75.4 / 77.8
+//   inverse    11.9 / 8.7  31.0 / 23.3 39.2 / 30.9 57.3 / 48.1 67.7 / 61.6 85.9 / 81.1
+//   Hadamard   13.4 / 9.2  40.7 / 27.5 49.6 / 38.0 73.6 / 61.7 91.8 / 74.3 116 / 95.0
+//   rescaling  11.1 / 9.3  29.6 / 25.6 35.8 / 35.4 53.3 / 57.1 65.6 / 68.8 84.2 / 87.8
+//   N = 2^15   24 rows     192         384         576         N = 2^17    24 rows     96          384
+//   forward    7.9 / 6.1   24.4 / 19.8 41.1 / 38.9 55.9 / 57.2             17.6 / 14.0 52.3 / 44.8 191 / 173
+//   inverse    9.3 / 6.3   26.0 / 20.5 44.6 / 36.8 60.7 / 57.3             22.0 / 14.8 62.2 / 43.7 219 / 170
+//   rescaling  9.3 / 6.7   27.8 / 24.0 45.7 / 44.0 63.1 / 64.9             19.5 / 16.4 56.3 / 52.6 209 / 196
+// and at N = 2^14 768 rows 43.1 / 38.3 and 40.8 / 34.3, 15 rows 7.9 / 5.0 and 8.7 / 5.2.
+bool two_pass(const hefx_params* p, NttMode mode, size_t rows) {
+    if (p->log2n < 14 || p->log2n > 17 || mode == MODE_FWD_HAD_INV || rows > (1u << 24)) return false;
+    if (p->cc_schedule != HEFX_CC_AUTO) return p->cc_schedule == HEFX_CC_TWO_PASS;
+    if (p->log2n == 17 || mode == MODE_HAD_INV || (p->log2n == 16 && mode == MODE_INV)) return true;
+    return (rows << p->log2n) >> 16 <= (mode == MODE_FWD ? 256u : mode == MODE_INV ? 320u : 144u);
+}
+
+cudaError_t launch_two_pass(const hefx_params* p, NttMode mode, const cc::KArgs& a, size_t rows, cudaStream_t stream) {
+    const bool lazy = p->max_prime < (1u << 28);
+    return p->log2n == 14 ? cc2::launch_14(mode, a, rows, stream, lazy)
+           : p->log2n == 15 ? cc2::launch_15(mode, a, rows, stream, lazy)
+           : p->log2n == 16 ? cc2::launch_16(mode, a, rows, stream, lazy)
+                            : cc2::launch_17(mode, a, rows, stream, lazy);
 }
 
 }  // namespace
@@ -31,32 +55,16 @@ cudaError_t encode_input_map(const hefx_params* p, const uint32_t* in, size_t ro
 
 cudaError_t launch_ntt_cc(const hefx_params* p, NttMode mode, const uint32_t* in, const uint32_t* had, uint32_t* out,
                           size_t rows, cudaStream_t stream) {
-    // AUTO takes the two-pass schedule where it measured faster than the clusters: up to 32
-    // rows (one polynomial of 24 limbs: 16.7 / 16.4 us against 20.7 / 20.5 us), and from one
-    // to one and a half waves of co-resident clusters, where the cluster kernel's second wave
-    // is mostly empty (96 rows: 34.1 / 31.7 us against 35.6 / 34.8 us; 120 rows: 43.3 / 39.9
-    // against 45.6 / 45.1 us); elsewhere the two are within a few percent and the single
-    // launch stays
-    bool two_pass = p->cc_schedule == HEFX_CC_TWO_PASS;
-    if (p->cc_schedule == HEFX_CC_AUTO && ntt_cc_2p_supported(p, mode)) {
-        constexpr size_t kTwoPassAutoRows = 32;
-        if (rows <= kTwoPassAutoRows) {
-            two_pass = true;
-        } else {
-            const size_t slots = (size_t)clusters16(p->ctx, mode, p->max_prime < (1u << 28));
-            two_pass = slots > 0 && rows > slots && 2 * rows <= 3 * slots;
-        }
-    }
-    if (two_pass && ntt_cc_2p_supported(p, mode)) return launch_ntt_cc_2p(p, mode, in, out, rows, stream);
     cc::KArgs a;
     memset(&a.tmap_in, 0, sizeof a.tmap_in);
     memset(&a.tmap_out, 0, sizeof a.tmap_out);
     a.err = p->d_err_cc;
-    if (mode == MODE_INV && rows > 0 && p->log2n >= 13) {
+    const bool tp = two_pass(p, mode, rows);
+    if (mode == MODE_INV && rows > 0 && p->log2n >= 13 && !tp) {
         cudaError_t e = encode_input_map(p, in, rows, &a.tmap_in);
         if (e != cudaSuccess) return e;
     }
-    if (mode == MODE_FWD && rows > 0 && p->log2n >= 13) {
+    if (mode == MODE_FWD && rows > 0 && p->log2n >= 13 && !tp) {
         cudaError_t e = encode_input_map(p, out, rows, &a.tmap_out);
         if (e != cudaSuccess) return e;
     }
@@ -71,7 +79,7 @@ cudaError_t launch_ntt_cc(const hefx_params* p, NttMode mode, const uint32_t* in
     a.L = p->nlimbs;
     a.in_rows = 0;
     if (rows == 0) return cudaSuccess;
-    return launch_dispatch(p, mode, a, rows, stream);
+    return tp ? launch_two_pass(p, mode, a, rows, stream) : launch_dispatch(p, mode, a, rows, stream);
 }
 
 cudaError_t launch_ntt_cc_rescale(const hefx_params* p, const uint32_t* in, uint32_t* out, size_t batch,
@@ -83,7 +91,8 @@ cudaError_t launch_ntt_cc_rescale(const hefx_params* p, const uint32_t* in, uint
     memset(&a.tmap_in, 0, sizeof a.tmap_in);
     memset(&a.tmap_out, 0, sizeof a.tmap_out);
     a.err = p->d_err_cc;
-    if (p->log2n >= 13) {
+    const bool tp = two_pass(p, MODE_RS_FWD, rows);
+    if (p->log2n >= 13 && !tp) {
         cudaError_t e = encode_input_map(p, out, rows, &a.tmap_out);
         if (e != cudaSuccess) return e;
     }
@@ -97,6 +106,7 @@ cudaError_t launch_ntt_cc_rescale(const hefx_params* p, const uint32_t* in, uint
     a.rows = (uint32_t)rows;
     a.L = L - 1;
     a.in_rows = L;
+    if (tp) return launch_two_pass(p, MODE_RS_FWD, a, rows, stream);
     cudaError_t e = launch_dispatch(p, MODE_RS_FWD, a, rows, stream);
     if (e != cudaErrorNotSupported) return e;
     // not fused at this N: rescale into out, then the forward transform of its L - 1 limbs
@@ -132,7 +142,7 @@ cudaError_t launch_ntt_cc_rows(const hefx_params* p, NttMode mode, const RowDesc
     a.L = p->nlimbs;
     a.in_rows = 0;
     if (nrows == 0) return cudaSuccess;
-    return launch_dispatch(p, mode, a, nrows, stream);
+    return two_pass(p, mode, nrows) ? launch_two_pass(p, mode, a, nrows, stream) : launch_dispatch(p, mode, a, nrows, stream);
 }
 
 cudaError_t launch_dispatch(const hefx_params* p, NttMode mode, const cc::KArgs& a, size_t rows, cudaStream_t stream) {

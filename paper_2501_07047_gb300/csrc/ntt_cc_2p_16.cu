@@ -1,0 +1,12 @@
+// Two-pass transforms of N = 2^16 (the kernels are in ntt_cc_2p.cuh).
+#include "ntt_cc_2p.cuh"
+
+namespace hefx {
+namespace cc2 {
+
+cudaError_t launch_16(NttMode mode, const KArgs& a, size_t rows, cudaStream_t s, bool lazy) {
+    return launch_logn<16>(mode, a, rows, s, lazy);
+}
+
+}  // namespace cc2
+}  // namespace hefx
