@@ -169,7 +169,9 @@ hefx_status hefx_params_set_reduction(hefx_params* params, hefx_reduction ntt_re
  *    in L2 (forward up to 256 rows of 2^16 elements, inverse 320, rescaling forward 144), and at
  *    N = 2^17, for the inverse at N = 2^16 and for that of a Hadamard product always; else
  *    HEFX_CC_CLUSTER.
- * The second half of hefx_poly_mul and fused batch plans use the cluster schedule.  Errors:
+ * hefx_poly_mul's second half is the cluster forward transform, multiplying on its way out, and
+ * the two-pass inverse unless HEFX_CC_CLUSTER is set (at N = 2^14 up to 128 rows); fused batch plans
+ * use the cluster schedule.  Errors:
  * EINVAL (unknown schedule), EUNSUPPORTED (HEFX_CC_TWO_PASS at N != 2^16).  Not thread-safe with concurrent calls that use the same params.
  */
 typedef enum { HEFX_CC_AUTO = 0, HEFX_CC_CLUSTER = 1, HEFX_CC_TWO_PASS = 2 } hefx_cc_schedule;
@@ -585,7 +587,8 @@ hefx_status hefx_batch_plan_create(hefx_ctx* ctx, const hefx_job* jobs, size_t n
 void hefx_batch_plan_destroy(hefx_batch_plan* plan);
 
 /*
- * Kernel launches one hefx_batch_polymul of the plan makes (1 for the fused form).
+ * Transform launches one hefx_batch_polymul of the plan makes (1 for the fused form; a transform
+ * on the two-pass schedule counts once).
  */
 uint32_t hefx_batch_plan_launches(const hefx_batch_plan* plan);
 

@@ -421,8 +421,12 @@ hefx_status hefx_poly_mul(hefx_ctx* ctx, const hefx_params* p, const uint32_t* a
         if (e == cudaSuccess) e = launch(MODE_HAD_INV, c, c, c);
     } else {
         if (c == b) std::swap(a, b);  // the product commutes; keep b intact while c is written
-        e = launch(MODE_FWD, a, nullptr, c);                    // c = NTT(a)
-        if (e == cudaSuccess) e = launch(MODE_FWD_HAD_INV, b, c, c);  // c = INTT(NTT(b) o c)
+        if (p->log2n <= 13) {  // a CTA holds whole rows: one launch
+            e = launch(MODE_PRODUCT, a, b, c);
+        } else {
+            e = launch(MODE_FWD, a, nullptr, c);                    // c = NTT(a)
+            if (e == cudaSuccess) e = launch(MODE_FWD_HAD_INV, b, c, c);  // c = INTT(NTT(b) o c)
+        }
     }
     if (e != cudaSuccess) return cuda_fail(ctx, e, "hefx_poly_mul launch");
     return HEFX_OK;

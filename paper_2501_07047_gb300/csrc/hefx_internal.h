@@ -188,7 +188,11 @@ cudaError_t launch_pdl(void (*kern)(Params...), dim3 grid, dim3 block, size_t sm
 // Kernel launchers (return a CUDA error code; the host API maps it to hefx_status).
 // MODE_RS_FWD: NTT(Rescale(x)): the forward transform of q_0..q_{L-2} whose first pass reads
 // limb i and the last limb of the same coefficient-form polynomial and rescales on the way in.
-enum NttMode { MODE_FWD = 0, MODE_INV = 1, MODE_FWD_HAD_INV = 2, MODE_HAD_INV = 3, MODE_RS_FWD = 4 };
+// MODE_FWD_HAD (cluster schedule) and MODE_INV_R (two-pass) are MODE_FWD_HAD_INV in two halves: the
+// forward transform times `had`, a Montgomery product below 2q, and the inverse scaled by N^-1 2^32.
+// MODE_PRODUCT (rows of one CTA): out = in * had, both in coefficient form, in one launch.
+enum NttMode { MODE_FWD = 0, MODE_INV = 1, MODE_FWD_HAD_INV = 2, MODE_HAD_INV = 3, MODE_RS_FWD = 4, MODE_FWD_HAD = 5,
+               MODE_INV_R = 6, MODE_PRODUCT = 7 };
 
 cudaError_t launch_ntt_cc(const hefx_params* p, NttMode mode, const uint32_t* in, const uint32_t* had, uint32_t* out,
                           size_t rows, cudaStream_t stream);

@@ -28,7 +28,9 @@ namespace {
 //   rescaling  9.3 / 6.7   27.8 / 24.0 45.7 / 44.0 63.1 / 64.9             19.5 / 16.4 56.3 / 52.6 209 / 196
 // and at N = 2^14 768 rows 43.1 / 38.3 and 40.8 / 34.3, 15 rows 7.9 / 5.0 and 8.7 / 5.2.
 bool two_pass(const hefx_params* p, NttMode mode, size_t rows) {
-    if (p->log2n < 14 || p->log2n > 17 || mode == MODE_FWD_HAD_INV || rows > (1u << 24)) return false;
+    if (p->log2n < 14 || p->log2n > 17 || mode == MODE_FWD_HAD_INV || mode == MODE_PRODUCT ||
+        rows > (1u << 24))
+        return false;
     if (p->cc_schedule != HEFX_CC_AUTO) return p->cc_schedule == HEFX_CC_TWO_PASS;
     if (p->log2n == 17 || mode == MODE_HAD_INV || (p->log2n == 16 && mode == MODE_INV)) return true;
     return (rows << p->log2n) >> 16 <= (mode == MODE_FWD ? 256u : mode == MODE_INV ? 320u : 144u);
@@ -40,6 +42,25 @@ cudaError_t launch_two_pass(const hefx_params* p, NttMode mode, const cc::KArgs&
            : p->log2n == 15 ? cc2::launch_15(mode, a, rows, stream, lazy)
            : p->log2n == 16 ? cc2::launch_16(mode, a, rows, stream, lazy)
                             : cc2::launch_17(mode, a, rows, stream, lazy);
+}
+
+// The product's second half, INTT(NTT(b) o c) with c in the output, as the cluster forward transform
+// that multiplies on its way out and the two-pass inverse, instead of one cluster launch with two
+// cross-CTA steps.  The whole product of two polynomials, us, one launch / this:
+//   N = 2^17   1 row 29.3 / 25.5   24 rows 55.1 / 51.2   96 rows 163 / 149
+//   N = 2^16   1 row 21.0 / 18.9   48 rows 44.0 / 44.7   96 rows 80.1 / 75.4   384 rows 249 / 244
+//   N = 2^15   1 row 19.8 / 17.4   96 rows 38.7 / 38.4   192 rows 71.3 / 67.9  384 rows 123 / 121
+//   N = 2^14   1 row 19.5 / 17.2   96 rows 26.8 / 26.1   192 rows 37.0 / 37.3  768 rows 117 / 118
+bool halves(const hefx_params* p, NttMode mode, size_t rows) {
+    return mode == MODE_FWD_HAD_INV && p->log2n >= 14 && p->log2n <= 17 && p->cc_schedule != HEFX_CC_CLUSTER &&
+           rows <= (p->log2n == 14 ? 128u : 1u << 24);
+}
+
+cudaError_t launch_halves(const hefx_params* p, cc::KArgs& a, size_t rows, cudaStream_t stream) {
+    cudaError_t e = launch_dispatch(p, MODE_FWD_HAD, a, rows, stream);
+    if (e != cudaSuccess) return e;
+    a.in = a.out;
+    return launch_two_pass(p, MODE_INV_R, a, rows, stream);
 }
 
 }  // namespace
@@ -79,6 +100,7 @@ cudaError_t launch_ntt_cc(const hefx_params* p, NttMode mode, const uint32_t* in
     a.L = p->nlimbs;
     a.in_rows = 0;
     if (rows == 0) return cudaSuccess;
+    if (halves(p, mode, rows)) return launch_halves(p, a, rows, stream);
     return tp ? launch_two_pass(p, mode, a, rows, stream) : launch_dispatch(p, mode, a, rows, stream);
 }
 

@@ -401,14 +401,16 @@ __global__ void __launch_bounds__(32, SM_WARPS) block_kernel(const __grid_consta
 
 template <int LOGN, int MODE, int F, int SMALL>
 cudaError_t launch_pair_t(const KArgs& a, size_t rows, cudaStream_t s) {
-    constexpr bool INV = MODE == MODE_INV || MODE == MODE_HAD_INV;
+    constexpr bool INV = MODE != MODE_FWD && MODE != MODE_RS_FWD;
+    // the scale N^-1 2^32 is the strided pass's only difference, the product the block pass's
+    constexpr int MS = MODE == MODE_INV_R ? MODE_HAD_INV : MODE, MB = MODE == MODE_INV_R ? MODE_INV : MODE;
     const dim3 gs((unsigned)(rows * Strided<LOGN, SMALL>::PARTS)), gb((unsigned)(rows << (LOGN - LOGB)));
     if (!INV) {
-        cudaError_t e = launch_pdl(strided_kernel<LOGN, MODE, F, SMALL>, gs, dim3(THREADS), 0, s, a);
-        return e != cudaSuccess ? e : launch_pdl(block_kernel<LOGN, MODE, F>, gb, dim3(32), 0, s, a);
+        cudaError_t e = launch_pdl(strided_kernel<LOGN, MS, F, SMALL>, gs, dim3(THREADS), 0, s, a);
+        return e != cudaSuccess ? e : launch_pdl(block_kernel<LOGN, MB, F>, gb, dim3(32), 0, s, a);
     }
-    cudaError_t e = launch_pdl(block_kernel<LOGN, MODE, F>, gb, dim3(32), 0, s, a);
-    return e != cudaSuccess ? e : launch_pdl(strided_kernel<LOGN, MODE, F, SMALL>, gs, dim3(THREADS), 0, s, a);
+    cudaError_t e = launch_pdl(block_kernel<LOGN, MB, F>, gb, dim3(32), 0, s, a);
+    return e != cudaSuccess ? e : launch_pdl(strided_kernel<LOGN, MS, F, SMALL>, gs, dim3(THREADS), 0, s, a);
 }
 // SMALL, 32 elements per thread of the strided pass: twice the warps, half the serial chain, and two
 // warps per position at N = 2^16.  Forward up to 44 rows of 2^16 elements, the inverse forms to
@@ -435,6 +437,7 @@ cudaError_t launch_mode(NttMode mode, const KArgs& a, size_t rows, cudaStream_t 
         case MODE_FWD: return launch_pair<LOGN, MODE_FWD, F>(a, rows, s);
         case MODE_INV: return launch_pair<LOGN, MODE_INV, F>(a, rows, s);
         case MODE_HAD_INV: return launch_pair<LOGN, MODE_HAD_INV, F>(a, rows, s);
+        case MODE_INV_R: return launch_pair<LOGN, MODE_INV_R, F>(a, rows, s);
         case MODE_RS_FWD:
             if constexpr ((F & 1) == 0) return launch_pair<LOGN, MODE_RS_FWD, F>(a, rows, s);
             else return cudaErrorNotSupported;

@@ -7,8 +7,8 @@
 //    split over a cluster of P CTAs (P = 8 at N = 2^16: 32 KiB + padding and 128 threads
 //    per CTA, registers sized for five CTAs of different rows per SM, so that their load,
 //    compute and barrier phases overlap).  Each row is read from and written to HBM once
-//    per transform (512 KiB per N = 2^16 limb-NTT).  A CTA with N < 2^13 holds 2^13 / N
-//    rows.
+//    per transform (512 KiB per N = 2^16 limb-NTT).  A CTA with N < 2^13 holds up to
+//    2^13 / N rows (rows_per_cta).
 //  - With P > 1 the log2(P) stages whose butterflies pair elements of different CTAs run
 //    as one radix-P step through distributed shared memory: the forward transform computes
 //    them while loading (each position j' of the first N/P is owned by one thread of the
@@ -100,12 +100,20 @@ __device__ __forceinline__ int swz_elem(int j0, int k) {
 #define HEFX_CC_LOGPW_BATCH 1
 #endif
 #ifndef HEFX_CC_WIDE_MODES
-#define HEFX_CC_WIDE_MODES 0x1b
+#define HEFX_CC_WIDE_MODES 0x3b
 #endif
 
 // F & 16 selects the configuration of the fused batch kernel (every ring degree in CTAs of
 // 128 threads and 2^13 elements, clusters of 8: one row of 2^16, two of 2^15, four of 2^14, or
 // eight CTA-sized groups of smaller rows per cluster).
+// Rows of one CTA (N <= 2^13): the registers are sized for two CTAs per SM, and for three at N = 2^13
+// or with kDense, which launches of more than two CTAs per SM take at N = 2^11 and 2^12.  With
+// one (210 to 250 registers) a launch of several waves was latency-bound; with three a single CTA
+// loses to its spilled twiddles.  us, one / two / three CTAs per SM: forward 1536 rows of 2^12
+// 32.2 / 23.1 / 20.9 and of 2^13 42.3 / 42.3 / 35.6, their products 95.0 / 64.9 / 59.8 and 150 /
+// 115 / 101; the product of one row of 2^12 8.3 / 8.4 / 9.0, of 2^13 13.0 / 12.9 / 12.9.
+constexpr int kDense = 512;
+
 template <int LOGN, int F = 0>
 struct Cfg {
     static constexpr int logP =
@@ -125,7 +133,7 @@ struct Cfg {
     static constexpr int threads = unified        ? 128
                                    : LOGN >= 17   ? HEFX_CC_THREADS17
                                    : small_split ? HEFX_CC_SPLIT_THREADS : (elems >= (1 << 14) ? 512 : 256);
-    static constexpr int minb = unified ? 5 : LOGN >= 17 ? HEFX_CC_MINB17 : small_split ? HEFX_CC_SPLIT_MINB : 1;
+    static constexpr int minb = unified ? 5 : LOGN >= 17 ? HEFX_CC_MINB17 : small_split ? HEFX_CC_SPLIT_MINB : LOGN == 13 || (F & kDense) != 0 ? 3 : 2;
     static constexpr int smem_bytes = elems * 4;
     static constexpr int S = logm;                  // stages run inside the CTA
     static constexpr int r_small = S < 5 ? S : 5;   // pass over the smallest strides
@@ -154,8 +162,13 @@ struct KArgs {
     const RowDesc* desc;  // per-row pointers and limb (batched jobs), or null: [rows][N] layout
     uint32_t rows;
     uint32_t L;
+    uint32_t rpc;      // rows per CTA of the unsplit kernels, 1 .. Cfg::rows
     uint32_t in_rows;  // MODE_RS_FWD: input rows per polynomial (the output has L = in_rows - 1)
 };
+
+// Flag bits of F in the one-launch product (MODE_PRODUCT): operands are written earlier in the same
+// launch; and its second half, whose input is a.had and whose Hadamard operand is a.out.
+constexpr int kFresh = 128, kSecond = 256;
 
 // Row r's input / Hadamard operand / output and limb, from the descriptor list when there
 // is one, else from the contiguous [batch][L][N] layout.
@@ -163,12 +176,12 @@ struct KArgs {
 template <int N, int F>
 __device__ __forceinline__ const uint32_t* row_in(const KArgs& a, uint32_t r) {
     if constexpr ((F & 1) != 0) return a.desc[r].in;
-    else return a.in + (size_t)r * N;
+    else return ((F & kSecond) != 0 ? a.had : a.in) + (size_t)r * N;
 }
 template <int N, int F>
 __device__ __forceinline__ const uint32_t* row_had(const KArgs& a, uint32_t r) {
     if constexpr ((F & 1) != 0) return a.desc[r].had;
-    else return a.had + (size_t)r * N;
+    else return ((F & kSecond) != 0 ? a.out : a.had) + (size_t)r * N;
 }
 template <int N, int F>
 __device__ __forceinline__ uint32_t* row_out(const KArgs& a, uint32_t r) {
@@ -202,7 +215,7 @@ __device__ __forceinline__ const uint2* row_twi(const KArgs& a, uint32_t r) {
 // same launch, so it takes the coherent path (L2) instead of the read-only one.
 template <int F, typename T>
 __device__ __forceinline__ T ld_had(const T* p) {
-    if constexpr ((F & 16) != 0) return __ldcg(p);
+    if constexpr ((F & (16 | kFresh)) != 0) return __ldcg(p);
     else return __ldg(p);
 }
 
@@ -246,8 +259,7 @@ __device__ __forceinline__ void load_elems(uint32_t (&x)[1 << R], const uint32_t
             for (int k = 0; k < (1 << R); ++k) x[k] = sm[swz_elem<R, logs, C::rows>(j0, k)];
         }
     } else {
-        const bool valid = row < sg.nrows;
-        const uint32_t grow_r = valid ? sg.row0 + row : sg.row0;
+        const uint32_t grow_r = sg.row0 + row;
         const uint32_t* rin = row_in<N, F>(a, grow_r);
         const uint32_t* rhad = SRC == SRC_GLOBAL_HAD ? row_had<N, F>(a, grow_r) : nullptr;
         if constexpr (logs == 0 && R >= 2) {
@@ -255,9 +267,9 @@ __device__ __forceinline__ void load_elems(uint32_t (&x)[1 << R], const uint32_t
             const uint4* hs = reinterpret_cast<const uint4*>(rhad + sg.gbase + jb);
 #pragma unroll
             for (int k = 0; k < (1 << R); k += 4) {
-                uint4 v = valid ? ld_had<F>(src + k / 4) : make_uint4(0, 0, 0, 0);
+                uint4 v = ld_had<F>(src + k / 4);
                 if constexpr (SRC == SRC_GLOBAL_HAD) {
-                    const uint4 h = valid ? ld_had<F>(hs + k / 4) : make_uint4(0, 0, 0, 0);
+                    const uint4 h = ld_had<F>(hs + k / 4);
                     v.x = mul_mont_lazy(v.x, h.x, lc.q, lc.qinv_neg);
                     v.y = mul_mont_lazy(v.y, h.y, lc.q, lc.qinv_neg);
                     v.z = mul_mont_lazy(v.z, h.z, lc.q, lc.qinv_neg);
@@ -272,8 +284,8 @@ __device__ __forceinline__ void load_elems(uint32_t (&x)[1 << R], const uint32_t
 #pragma unroll
             for (int k = 0; k < (1 << R); ++k) {
                 const size_t g = sg.gbase + jb + (k << logs);
-                uint32_t v = valid ? ld_had<F>(rin + g) : 0u;
-                if constexpr (SRC == SRC_GLOBAL_HAD) v = mul_mont_lazy(v, valid ? ld_had<F>(rhad + g) : 0u, lc.q, lc.qinv_neg);
+                uint32_t v = ld_had<F>(rin + g);
+                if constexpr (SRC == SRC_GLOBAL_HAD) v = mul_mont_lazy(v, ld_had<F>(rhad + g), lc.q, lc.qinv_neg);
                 x[k] = v;
             }
         }
@@ -646,14 +658,14 @@ __device__ __forceinline__ void fwd_pass(uint32_t* sm, const Seg& sg, const KArg
             store_elems<R, LOGN, logtl, DST, F>(x, sm, a, sg, 0, jb, lc);
         }
     } else {
-        for (int u = threadIdx.x; u < C::rows * nsub; u += C::threads) {
+        for (int u = threadIdx.x; u < (C::rows == 1 ? 1 : sg.nrows) * nsub; u += C::threads) {
             const int row = C::rows == 1 ? 0 : u >> lognsub;
             const int uu = u & (nsub - 1);
             const int j_lo = uu & ((1 << logtl) - 1);
             const int j_hi = uu >> logtl;
             const int jb = (j_hi << (logtl + R)) + j_lo;
             const uint32_t g0 = (sg.gbase >> (logtl + R)) + (uint32_t)j_hi;
-            const uint32_t rr = row < sg.nrows ? sg.row0 + row : sg.row0;
+            const uint32_t rr = sg.row0 + row;
             const LimbConst& lc = row_lc<F>(a, rr);
             const uint2* tw = row_twf<N, F>(a, rr);
             uint32_t x[1 << R];
@@ -708,13 +720,13 @@ __device__ __forceinline__ void inv_pass(uint32_t* sm, const Seg& sg, const KArg
             store_elems<R, LOGN, e0, DST, F>(x, sm, a, sg, 0, jb, lc);
         }
     } else {
-        for (int u = threadIdx.x; u < C::rows * nsub; u += C::threads) {
+        for (int u = threadIdx.x; u < (C::rows == 1 ? 1 : sg.nrows) * nsub; u += C::threads) {
             const int row = C::rows == 1 ? 0 : u >> lognsub;
             const int uu = u & (nsub - 1);
             const int j_lo = uu & ((1 << e0) - 1);
             const int j_hi = uu >> e0;
             const int jb = (j_hi << (e0 + R)) + j_lo;
-            const uint32_t rr = row < sg.nrows ? sg.row0 + row : sg.row0;
+            const uint32_t rr = sg.row0 + row;
             const LimbConst& lc = row_lc<F>(a, rr);
             const uint2* tw = row_twi<N, F>(a, rr);
             uint32_t x[1 << R];
@@ -735,21 +747,25 @@ __device__ __forceinline__ void fwd_had_inv_pass(uint32_t* sm, const Seg& sg, co
     constexpr int lognsub = C::logm - R;
     constexpr int nsub = 1 << lognsub;
     static_assert(LOGN - s0 - R == 0, "the fused pass covers the smallest strides");
-    for (int u = threadIdx.x; u < C::rows * nsub; u += C::threads) {
+    for (int u = threadIdx.x; u < (C::rows == 1 ? 1 : sg.nrows) * nsub; u += C::threads) {
         const int row = C::rows == 1 ? 0 : u >> lognsub;
         const int j_hi = u & (nsub - 1);
         const int jb = j_hi << R;
         const uint32_t g0 = (sg.gbase >> R) + (uint32_t)j_hi;
-        const uint32_t rr = row < sg.nrows ? sg.row0 + row : sg.row0;
+        const uint32_t rr = sg.row0 + row;
         const LimbConst& lc = row_lc<F>(a, rr);
         uint32_t x[1 << R];
+        const uint4* hs = reinterpret_cast<const uint4*>(row_had<N, F>(a, rr) + sg.gbase + jb);
+        // the operand is requested before the forward stages (192 rows of 2^16: 142.4 -> 138.5 us a product)
+        constexpr int HV = (1 << R) / 4 > 0 ? (1 << R) / 4 : 1;
+        uint4 hh[HV];
+#pragma unroll
+        for (int k = 0; k < HV; ++k) hh[k] = ld_had<F>(hs + k);
         load_elems<R, LOGN, 0, SRC, F>(x, sm, a, sg, row, jb, lc);
         fwd_stages<R, LOGN, s0, F | kLooseOut>(x, g0, row_twf<N, F>(a, rr), lc);
-        const bool valid = row < sg.nrows;
-        const uint4* hs = reinterpret_cast<const uint4*>(row_had<N, F>(a, valid ? sg.row0 + row : sg.row0) + sg.gbase + jb);
 #pragma unroll
         for (int k = 0; k < (1 << R); k += 4) {
-            const uint4 h = valid ? ld_had<F>(hs + k / 4) : make_uint4(0, 0, 0, 0);
+            const uint4 h = hh[k / 4];
             x[k] = mul_mont_lazy(x[k], h.x, lc.q, lc.qinv_neg);
             x[k + 1] = mul_mont_lazy(x[k + 1], h.y, lc.q, lc.qinv_neg);
             x[k + 2] = mul_mont_lazy(x[k + 2], h.z, lc.q, lc.qinv_neg);
@@ -959,7 +975,7 @@ __host__ __device__ constexpr bool tma_input() {
 // reduces into the swizzled buffer, one thread stores it as 256-line boxes).
 template <int LOGN, int MODE, int F>
 __host__ __device__ constexpr bool tma_output() {
-    return (MODE == MODE_FWD || MODE == MODE_RS_FWD) && (F & 1) == 0 && LOGN >= 13;
+    return (MODE == MODE_FWD || MODE == MODE_RS_FWD) && (F & (1 | kFresh)) == 0 && LOGN >= 13;
 }
 template <int LOGN, int MODE, int F>
 __host__ __device__ constexpr bool uses_tma() {
@@ -968,21 +984,35 @@ __host__ __device__ constexpr bool uses_tma() {
 
 // Where TMA does not apply (row lists, N < 2^13) the first inverse pass and the last forward
 // pass still move whole lines: the CTA copies its rows between global and shared memory with
-// lane-consecutive 16-byte accesses (the Hadamard product, if any, applied on the way in).
+// lane-consecutive 16-byte accesses (the Hadamard product, if any, applied on the way in), four or
+// eight of them in flight (inverse of a Hadamard product, 900 rows of 2^13: 31.8 -> 28.5 us).
 template <int LOGN, int F, bool HAD>
 __device__ __forceinline__ void copy_in(uint32_t* sm, const Seg& sg, const KArgs& a) {
     using C = Cfg<LOGN, F>;
-    constexpr int N = 1 << LOGN;
-    for (int idx = threadIdx.x * 4; idx < sg.nrows * C::m; idx += C::threads * 4) {
-        const int row = idx >> C::logm, i = idx & (C::m - 1);
-        uint4 v = ld_had<F>(reinterpret_cast<const uint4*>(row_in<N, F>(a, sg.row0 + row) + sg.gbase + i));
-        if constexpr (HAD) {
-            const uint4 h = ld_had<F>(reinterpret_cast<const uint4*>(row_had<N, F>(a, sg.row0 + row) + sg.gbase + i));
-            const LimbConst& lc = row_lc<F>(a, sg.row0 + row);
-            v = make_uint4(mul_mont_lazy(v.x, h.x, lc.q, lc.qinv_neg), mul_mont_lazy(v.y, h.y, lc.q, lc.qinv_neg),
-                           mul_mont_lazy(v.z, h.z, lc.q, lc.qinv_neg), mul_mont_lazy(v.w, h.w, lc.q, lc.qinv_neg));
+    constexpr int N = 1 << LOGN, STEP = C::threads * 4;
+    constexpr int U = !C::unified && (C::rows == 1 || (!HAD && (F & kDense) == 0)) ? 8 : 4;  // what the registers hold
+    const int total = (C::rows == 1 ? 1 : sg.nrows) * C::m;
+    // U accesses (of each operand) in flight per thread
+    for (int idx0 = threadIdx.x * 4; idx0 < total; idx0 += U * STEP) {
+        uint4 v[U], h[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int idx = idx0 + u * STEP, row = idx >> C::logm, i = idx & (C::m - 1);
+            if (idx >= total) break;
+            v[u] = ld_had<F>(reinterpret_cast<const uint4*>(row_in<N, F>(a, sg.row0 + row) + sg.gbase + i));
+            if constexpr (HAD) h[u] = ld_had<F>(reinterpret_cast<const uint4*>(row_had<N, F>(a, sg.row0 + row) + sg.gbase + i));
         }
-        *reinterpret_cast<uint4*>(&sm[swz(row * C::m + i)]) = v;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int idx = idx0 + u * STEP, row = idx >> C::logm, i = idx & (C::m - 1);
+            if (idx >= total) break;
+            if constexpr (HAD) {
+                const LimbConst& lc = row_lc<F>(a, sg.row0 + row);
+                v[u] = make_uint4(mul_mont_lazy(v[u].x, h[u].x, lc.q, lc.qinv_neg), mul_mont_lazy(v[u].y, h[u].y, lc.q, lc.qinv_neg),
+                                  mul_mont_lazy(v[u].z, h[u].z, lc.q, lc.qinv_neg), mul_mont_lazy(v[u].w, h[u].w, lc.q, lc.qinv_neg));
+            }
+            *reinterpret_cast<uint4*>(&sm[swz(row * C::m + i)]) = v[u];
+        }
     }
     __syncthreads();
 }
@@ -992,10 +1022,33 @@ __device__ __forceinline__ void copy_out(const uint32_t* sm, const Seg& sg, cons
     using C = Cfg<LOGN, F>;
     constexpr int N = 1 << LOGN;
     __syncthreads();
-    for (int idx = threadIdx.x * 4; idx < sg.nrows * C::m; idx += C::threads * 4) {
+    for (int idx = threadIdx.x * 4; idx < (C::rows == 1 ? 1 : sg.nrows) * C::m; idx += C::threads * 4) {
         const int row = idx >> C::logm, i = idx & (C::m - 1);
-        *reinterpret_cast<uint4*>(row_out<N, F>(a, sg.row0 + row) + sg.gbase + i) =
-            *reinterpret_cast<const uint4*>(&sm[swz(row * C::m + i)]);
+        uint4 v = *reinterpret_cast<const uint4*>(&sm[swz(row * C::m + i)]);
+        *reinterpret_cast<uint4*>(row_out<N, F>(a, sg.row0 + row) + sg.gbase + i) = v;
+    }
+}
+
+// The CTA's part of a split row times the Hadamard operand (Montgomery) on the way out.  The operand
+// is requested whole before the last barrier: loaded as needed, its sixteen round trips made the
+// product of 192 rows of 2^16 147 us instead of 132.5.
+template <int LOGN, int F>
+__device__ __forceinline__ void copy_out_had(const uint32_t* sm, const Seg& sg, const KArgs& a) {
+    using C = Cfg<LOGN, F>;
+    constexpr int N = 1 << LOGN, ITERS = C::m / (C::threads * 4);
+    const uint4* had = reinterpret_cast<const uint4*>(row_had<N, F>(a, sg.row0) + sg.gbase) + threadIdx.x;
+    uint4* out = reinterpret_cast<uint4*>(row_out<N, F>(a, sg.row0) + sg.gbase) + threadIdx.x;
+    const LimbConst& lc = row_lc<F>(a, sg.row0);
+    uint4 h[ITERS];
+#pragma unroll
+    for (int k = 0; k < ITERS; ++k) h[k] = __ldcg(had + k * C::threads);
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < ITERS; ++k) {
+        const uint4 v = *reinterpret_cast<const uint4*>(&sm[swz((k * C::threads + (int)threadIdx.x) * 4)]);
+        out[k * C::threads] =
+            make_uint4(mul_mont_lazy(v.x, h[k].x, lc.q, lc.qinv_neg), mul_mont_lazy(v.y, h[k].y, lc.q, lc.qinv_neg),
+                       mul_mont_lazy(v.z, h[k].z, lc.q, lc.qinv_neg), mul_mont_lazy(v.w, h[k].w, lc.q, lc.qinv_neg));
     }
 }
 
@@ -1049,7 +1102,7 @@ __device__ __forceinline__ void run_task(uint32_t* sm, const Seg& sg, const KArg
     constexpr int S_SMALL = LOGN - RS;            // first stage of the smallest-stride pass
     constexpr int FW = F | (((HEFX_CC_WIDE_MODES >> MODE) & 1) ? kWide : 0);  // F of the big-stride passes
 
-    if constexpr (MODE == MODE_FWD || MODE == MODE_RS_FWD) {
+    if constexpr (MODE == MODE_FWD || MODE == MODE_RS_FWD || MODE == MODE_FWD_HAD) {
         constexpr bool TMA = tma_output<LOGN, MODE, F>();
         static_assert(MODE == MODE_FWD || C::split, "the rescaling load is the cross-CTA pass");
         if constexpr (C::split) fwd_cross_pass<LOGN, F, MODE == MODE_RS_FWD>(sm, sg, a);
@@ -1058,6 +1111,11 @@ __device__ __forceinline__ void run_task(uint32_t* sm, const Seg& sg, const KArg
             fwd_pass<RS, LOGN, S_FIRST, C::split ? SRC_SMEM : SRC_GLOBAL, DST_GLOBAL_REDUCE, F>(sm, sg, a);
         } else {
             fwd_big<LOGN, 0, S_FIRST, FW>(sm, sg, a);
+            if constexpr (MODE == MODE_FWD_HAD) {
+                fwd_pass<RS, LOGN, S_SMALL, SRC_SMEM, DST_SMEM, F | kLooseOut>(sm, sg, a);
+                copy_out_had<LOGN, F>(sm, sg, a);
+                return;
+            }
             fwd_pass<RS, LOGN, S_SMALL, SRC_SMEM, DST_SMEM_REDUCE, F>(sm, sg, a);
             if constexpr (TMA) store_part_tma<LOGN>(sm, sg, a);
             else copy_out<LOGN, F>(sm, sg, a);
@@ -1091,7 +1149,8 @@ __device__ __forceinline__ void run_task(uint32_t* sm, const Seg& sg, const KArg
 }
 
 template <int LOGN, int MODE, int F>
-__global__ void __launch_bounds__(Cfg<LOGN, F>::threads, Cfg<LOGN, F>::minb) ntt_cc_kernel(const __grid_constant__ KArgs a) {
+__global__ void __launch_bounds__(Cfg<LOGN, F>::threads, LOGN == 13 && MODE == MODE_HAD_INV ? 2 : Cfg<LOGN, F>::minb)
+    ntt_cc_kernel(const __grid_constant__ KArgs a) {
     using C = Cfg<LOGN, F>;
     extern __shared__ __align__(16) uint32_t sm_raw[];
     __shared__ uint64_t tma_bar;
@@ -1110,8 +1169,8 @@ __global__ void __launch_bounds__(Cfg<LOGN, F>::threads, Cfg<LOGN, F>::minb) ntt
     // programmatic dependent launch: every global access (and every cluster access) is below
     griddep_wait();
     // persistent: each CTA (or cluster of P CTAs) walks a strided sequence of tasks; a task
-    // is one row (split N) or C::rows rows
-    const uint32_t ntasks = C::split ? a.rows : (a.rows + C::rows - 1) / C::rows;
+    // is one row (split N) or a.rpc rows
+    const uint32_t ntasks = C::split ? a.rows : (a.rows + a.rpc - 1) / a.rpc;
     const uint32_t first = blockIdx.x >> C::logP;
     const uint32_t stride = gridDim.x >> C::logP;
     for (uint32_t task = first; task < ntasks; task += stride) {
@@ -1121,9 +1180,9 @@ __global__ void __launch_bounds__(Cfg<LOGN, F>::threads, Cfg<LOGN, F>::minb) ntt
             sg.part = blockIdx.x & (C::P - 1);  // == rank in the cluster
             sg.nrows = 1;
         } else {
-            sg.row0 = task * C::rows;
+            sg.row0 = task * a.rpc;
             sg.part = 0;
-            sg.nrows = (int)min((uint32_t)C::rows, a.rows - sg.row0);
+            sg.nrows = (int)min(a.rpc, a.rows - sg.row0);
         }
         sg.gbase = sg.part * C::m;
         sg.rbase = 0;
@@ -1131,6 +1190,40 @@ __global__ void __launch_bounds__(Cfg<LOGN, F>::threads, Cfg<LOGN, F>::minb) ntt
         // shared memory is reused by the next task; with a split row the peers write into it
         if (task + stride < ntasks) sync_all<C::split>();
     }
+}
+
+// Rows per CTA of an unsplit launch: the number that leaves the busiest SM the fewest rows, the larger of
+// equals (its CTA loads the twiddles once).  A CTA that always took 2^13 elements left most SMs idle
+// on few rows, and ran its passes over rows that were not there.  us, before / after: 3 rows of
+// 2^11 4.7 / 2.6 and their product 13.1 / 7.1, 48 rows of 2^12 5.8 / 3.7 and 16.3 / 10.2, 240 rows
+// of 2^10 4.3 / 2.9 and 11.6 / 8.3, 16000 rows of 2^3 5.0 / 1.7.
+inline uint32_t rows_per_cta(size_t rows, size_t most) {
+    constexpr size_t SMS = 152;
+    const size_t k0 = std::max<size_t>(1, (rows + SMS * most - 1) / (SMS * most));  // CTAs of `most` rows on an SM
+    if (k0 > 4) return (uint32_t)most;
+    size_t best = most, load = k0 * most;
+    for (size_t k = k0; k <= k0 + 2; ++k) {
+        const size_t r = (rows + SMS * k - 1) / (SMS * k);
+        if (k * r < load) best = r, load = k * r;
+    }
+    return (uint32_t)best;
+}
+
+// The product of rows that one CTA holds, both halves in one launch: c = NTT(a), read back from L2 by
+// the second half.  Against two launches (us): one row of 2^12 9.8 / 8.4, 8 rows of 2^13 14.6 /
+// 13.4, 1536 rows of 2^12 61.3 / 59.8.
+template <int LOGN, int F>
+__global__ void __launch_bounds__(Cfg<LOGN, F>::threads, Cfg<LOGN, F>::minb) ntt_cc_product_kernel(const __grid_constant__ KArgs a) {
+    using C = Cfg<LOGN, F>;
+    extern __shared__ __align__(16) uint32_t sm_raw[];
+    uint32_t unused_phase = 0;
+    Seg sg = {};
+    sg.row0 = blockIdx.x * a.rpc;
+    sg.nrows = (int)min(a.rpc, a.rows - sg.row0);
+    griddep_wait();
+    run_task<LOGN, MODE_FWD, F | kFresh>(sm_raw, sg, a, nullptr, unused_phase);
+    __syncthreads();
+    run_task<LOGN, MODE_FWD_HAD_INV, F | kFresh | kSecond>(sm_raw, sg, a, nullptr, unused_phase);
 }
 
 // rows == 0: set the kernel's attributes only (done before a stream capture).
@@ -1170,9 +1263,11 @@ cudaError_t launch_one(const KArgs& a, size_t rows, cudaStream_t stream) {
         attr_set[dev & 63] = true;
     }
     if (rows == 0) return cudaSuccess;
-    const size_t groups = C::split ? rows : (rows + C::rows - 1) / C::rows;
+    KArgs b = a;
+    b.rpc = rows_per_cta(rows, C::rows);
+    const size_t groups = C::split ? rows : (rows + b.rpc - 1) / b.rpc;
     cfg.gridDim = dim3((unsigned)(C::P * groups));
-    return cudaLaunchKernelEx(&cfg, kern, a);
+    return cudaLaunchKernelEx(&cfg, kern, b);
 }
 
 template <int LOGN, int F>
@@ -1180,7 +1275,21 @@ cudaError_t launch_mode_d(NttMode mode, const KArgs& a, size_t rows, cudaStream_
     switch (mode) {
         case MODE_FWD: return launch_one<LOGN, MODE_FWD, F>(a, rows, s);
         case MODE_INV: return launch_one<LOGN, MODE_INV, F>(a, rows, s);
-        case MODE_FWD_HAD_INV: return launch_one<LOGN, MODE_FWD_HAD_INV, F>(a, rows, s);
+        case MODE_FWD_HAD_INV:
+            if constexpr (Cfg<LOGN>::split || (F & 1) != 0) return launch_one<LOGN, MODE_FWD_HAD_INV, F>(a, rows, s);
+            else return cudaErrorNotSupported;  // MODE_PRODUCT
+        case MODE_PRODUCT:
+            if constexpr (!Cfg<LOGN>::split && (F & 1) == 0) {
+                using C = Cfg<LOGN, F>;
+                static_assert(C::smem_bytes <= 48 << 10, "no attribute to set");
+                KArgs b = a;
+                b.rpc = rows_per_cta(rows, C::rows);
+                return launch_pdl(ntt_cc_product_kernel<LOGN, F>, dim3((unsigned)((rows + b.rpc - 1) / b.rpc)),
+                                  dim3(C::threads), C::smem_bytes, s, b);
+            } else return cudaErrorNotSupported;
+        case MODE_FWD_HAD:
+            if constexpr (Cfg<LOGN>::split) return launch_one<LOGN, MODE_FWD_HAD, F>(a, rows, s);
+            else return cudaErrorNotSupported;
         case MODE_RS_FWD:
             if constexpr ((F & 1) == 0 && Cfg<LOGN>::split) return launch_one<LOGN, MODE_RS_FWD, F>(a, rows, s);
             else return cudaErrorNotSupported;
@@ -1191,6 +1300,13 @@ cudaError_t launch_mode_d(NttMode mode, const KArgs& a, size_t rows, cudaStream_
 // lazy: every modulus of the parameter set is below 2^28
 template <int LOGN>
 cudaError_t launch_mode(NttMode mode, const KArgs& a, size_t rows, cudaStream_t s, bool lazy) {
+    if constexpr (LOGN == 11 || LOGN == 12) {
+        if (rows > 2 * 152 * (size_t)rows_per_cta(rows, Cfg<LOGN>::rows)) {
+            if (a.desc)
+                return lazy ? launch_mode_d<LOGN, kDense | 3>(mode, a, rows, s) : launch_mode_d<LOGN, kDense | 1>(mode, a, rows, s);
+            return lazy ? launch_mode_d<LOGN, kDense | 2>(mode, a, rows, s) : launch_mode_d<LOGN, kDense>(mode, a, rows, s);
+        }
+    }
     if (a.desc) return lazy ? launch_mode_d<LOGN, 3>(mode, a, rows, s) : launch_mode_d<LOGN, 1>(mode, a, rows, s);
     return lazy ? launch_mode_d<LOGN, 2>(mode, a, rows, s) : launch_mode_d<LOGN, 0>(mode, a, rows, s);
 }
