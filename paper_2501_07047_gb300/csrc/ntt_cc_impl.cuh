@@ -107,7 +107,7 @@ __device__ __forceinline__ int swz_elem(int j0, int k) {
 // 128 threads and 2^13 elements, clusters of 8: one row of 2^16, two of 2^15, four of 2^14, or
 // eight CTA-sized groups of smaller rows per cluster).
 // Rows of one CTA (N <= 2^13): the registers are sized for two CTAs per SM, and for three at N = 2^13
-// or with kDense, which launches of more than two CTAs per SM take at N = 2^11 and 2^12.  With
+// (but for row lists) or with kDense, which launches of more than two CTAs per SM take at N = 2^11 and 2^12.  With
 // one (210 to 250 registers) a launch of several waves was latency-bound; with three a single CTA
 // loses to its spilled twiddles.  us, one / two / three CTAs per SM: forward 1536 rows of 2^12
 // 32.2 / 23.1 / 20.9 and of 2^13 42.3 / 42.3 / 35.6, their products 95.0 / 64.9 / 59.8 and 150 /
@@ -133,7 +133,8 @@ struct Cfg {
     static constexpr int threads = unified        ? 128
                                    : LOGN >= 17   ? HEFX_CC_THREADS17
                                    : small_split ? HEFX_CC_SPLIT_THREADS : (elems >= (1 << 14) ? 512 : 256);
-    static constexpr int minb = unified ? 5 : LOGN >= 17 ? HEFX_CC_MINB17 : small_split ? HEFX_CC_SPLIT_MINB : LOGN == 13 || (F & kDense) != 0 ? 3 : 2;
+    static constexpr int minb = unified ? 5 : LOGN >= 17 ? HEFX_CC_MINB17 : small_split ? HEFX_CC_SPLIT_MINB
+                                         : (LOGN == 13 && (F & 1) == 0) || (F & kDense) != 0 ? 3 : 2;
     static constexpr int smem_bytes = elems * 4;
     static constexpr int S = logm;                  // stages run inside the CTA
     static constexpr int r_small = S < 5 ? S : 5;   // pass over the smallest strides
