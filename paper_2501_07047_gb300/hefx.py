@@ -180,7 +180,7 @@ def hefx_params_set_reduction(ctx, params: int, ntt_red="shoup", vec_red="montgo
 
 def hefx_params_set_cc_schedule(ctx, params: int, schedule="auto") -> None:
     """Schedule of the contiguous CUDA-core transforms: "cluster" (one launch, 8-CTA clusters),
-    "two_pass" (N = 2^16: column pass + block pass through L2) or "auto"."""
+    "two_pass" (N = 2^16: strided pass + block pass through L2) or "auto"."""
     _check(ctx, load().hefx_params_set_cc_schedule(params, CC_SCHEDULES[schedule]))
 
 
