@@ -629,6 +629,15 @@ hefx_status hefx_stream_check(hefx_ctx* ctx, const hefx_params* params, void* st
  */
 hefx_status hefx_wait_check(hefx_ctx* ctx, const hefx_params* params, uint64_t limit_ns, int arrive, void* stream);
 
+/*
+ * The same check for a warp whose lanes must go on or give up together: lane i's barrier has
+ * completed when bit i of `lanes` is set, nothing ever arrives on the others'.  With every bit
+ * set the next hefx_stream_check returns HEFX_OK; otherwise the whole warp gives up after
+ * limit_ns, with the code of hefx_wait_check (a warp that split is recorded under another code).
+ */
+hefx_status hefx_wait_check_warp(hefx_ctx* ctx, const hefx_params* params, uint64_t limit_ns, uint32_t lanes,
+                                 void* stream);
+
 #ifdef __cplusplus
 }
 #endif

@@ -287,8 +287,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         Ring r = {0, 0};
         uint32_t used = 0;
         for (uint32_t t = blk; t < ntiles; t += nblk) {
-            const bool ok = tc::mbar_wait(&raw_empty[r.i], r.ph ^ 1u, err, tc::ERR_TIMEOUT_EMPTY);
-            if (!__all_sync(0xffffffffu, ok)) break;
+            if (!tc::mbar_wait_warp(&raw_empty[r.i], r.ph ^ 1u, err, tc::ERR_TIMEOUT_EMPTY)) break;
             uint8_t* dst = smem + a.lay.raw_off + r.i * a.lay.raw_bytes;
             if (lane == 0) {
                 // one 2D copy: 128 words x the map's box of rows (rows past a ragged digit go unused)
@@ -323,8 +322,8 @@ __global__ void __launch_bounds__(THREADS, 1)
         const uint32_t full = kc >> 6, rest = (kc & 63) >> 4;  // 64-column chunks of digits, steps of the last
         Ring ra = {0, 0}, rc = {0, 0};
         for (uint32_t t = blk; t < ntiles; t += nblk) {
-            if (!__all_sync(0xffffffffu, tc::mbar_wait(&a_full[ra.i], ra.ph, err, tc::ERR_TIMEOUT_FULL) &&
-                                             tc::mbar_wait(&acc_empty[rc.i], rc.ph ^ 1u, err, tc::ERR_TIMEOUT_ACC)))
+            if (!tc::mbar_wait_warp(&a_full[ra.i], ra.ph, err, tc::ERR_TIMEOUT_FULL) ||
+                !tc::mbar_wait_warp(&acc_empty[rc.i], rc.ph ^ 1u, err, tc::ERR_TIMEOUT_ACC))
                 break;
             tc::tc_fence_after();
             const uint64_t ab = a0 + ra.i * a_step;
@@ -357,8 +356,8 @@ __global__ void __launch_bounds__(THREADS, 1)
         rr.advance(group, stages);
         ra.advance(group, abufs);
         for (uint64_t t = blk + (uint64_t)group * nblk; t < ntiles; t += (uint64_t)producers * nblk) {
-            if (!tc::mbar_wait(&raw_full[rr.i], rr.ph, err, tc::ERR_TIMEOUT_FULL)) break;
-            if (!tc::mbar_wait(&a_empty[ra.i], ra.ph ^ 1u, err, tc::ERR_TIMEOUT_EMPTY)) break;
+            if (!tc::mbar_wait_warp(&raw_full[rr.i], rr.ph, err, tc::ERR_TIMEOUT_FULL)) break;
+            if (!tc::mbar_wait_warp(&a_empty[ra.i], ra.ph ^ 1u, err, tc::ERR_TIMEOUT_EMPTY)) break;
             const uint32_t* raw = reinterpret_cast<const uint32_t*>(smem + a.lay.raw_off + rr.i * a.lay.raw_bytes) + row;
             uint8_t* A = smem + ra.i * a.lay.a_bytes + row * 128;
             char* own = nullptr;  // ModUp copies the digit's own limbs
@@ -465,7 +464,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             if (j0 < Lp) group8(j0, std::false_type{});
         };
         for (uint64_t t = blk + (uint64_t)eg * nblk; t < ntiles; t += (uint64_t)epis * nblk) {
-            if (!tc::mbar_wait(&acc_full[rc.i], rc.ph, err, tc::ERR_TIMEOUT_ACC)) break;
+            if (!tc::mbar_wait_warp(&acc_full[rc.i], rc.ph, err, tc::ERR_TIMEOUT_ACC)) break;
             tc::tc_fence_after();
             const uint32_t cols = tmem + quad + rc.i * npad;
             epilogue((uint32_t)t, cols);

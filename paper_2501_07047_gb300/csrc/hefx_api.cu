@@ -1040,14 +1040,26 @@ hefx_status hefx_params_set_tensor_config(hefx_params* p, uint32_t log2r, uint32
     return HEFX_OK;
 }
 
-hefx_status hefx_wait_check(hefx_ctx* ctx, const hefx_params* p, uint64_t limit_ns, int arrive, void* stream) {
+static hefx_status wait_check_args(hefx_ctx* ctx, const hefx_params* p, uint64_t limit_ns) {
     if (!ctx) return HEFX_EINVAL;
     if (!p || p->ctx != ctx) return fail(ctx, HEFX_EINVAL, "params is null or belongs to another context");
     if (limit_ns > 2000000000ull) return fail(ctx, HEFX_EINVAL, "limit_ns above the 2 s wait limit of the kernels");
-    hefx_status st = use_device(ctx);
+    return use_device(ctx);
+}
+
+hefx_status hefx_wait_check(hefx_ctx* ctx, const hefx_params* p, uint64_t limit_ns, int arrive, void* stream) {
+    hefx_status st = wait_check_args(ctx, p, limit_ns);
     if (st != HEFX_OK) return st;
     cudaError_t e = launch_wait_check(p->d_err_cc, limit_ns, arrive, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "hefx_wait_check launch");
+    return HEFX_OK;
+}
+
+hefx_status hefx_wait_check_warp(hefx_ctx* ctx, const hefx_params* p, uint64_t limit_ns, uint32_t lanes, void* stream) {
+    hefx_status st = wait_check_args(ctx, p, limit_ns);
+    if (st != HEFX_OK) return st;
+    cudaError_t e = launch_wait_check_warp(p->d_err_cc, limit_ns, lanes, (cudaStream_t)stream);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "hefx_wait_check_warp launch");
     return HEFX_OK;
 }
 

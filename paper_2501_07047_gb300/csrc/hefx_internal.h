@@ -264,6 +264,7 @@ void tc_free(hefx_params* p);
 cudaError_t tc_check(const hefx_params* p, cudaStream_t stream, uint32_t* code);
 size_t noalloc_scratch_words();
 cudaError_t launch_wait_check(uint32_t* err, uint64_t limit_ns, int arrive, cudaStream_t stream);
+cudaError_t launch_wait_check_warp(uint32_t* err, uint64_t limit_ns, uint32_t lanes, cudaStream_t stream);
 // Read access to a serving plan's fields (hefx_api.cu) for the batched request (mult_batch.cu).
 struct MultPlanView {
     hefx_ctx* ctx;

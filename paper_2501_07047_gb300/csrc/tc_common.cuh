@@ -15,7 +15,7 @@ namespace tc {
 
 constexpr uint64_t kWaitLimitNs = 2000000000ull;  // 2 s
 
-enum : uint32_t { ERR_NONE = 0, ERR_TIMEOUT_FULL = 1, ERR_TIMEOUT_EMPTY = 2, ERR_TIMEOUT_ACC = 3, ERR_WAIT_CHECK = 32 };
+enum : uint32_t { ERR_NONE = 0, ERR_TIMEOUT_FULL = 1, ERR_TIMEOUT_EMPTY = 2, ERR_TIMEOUT_ACC = 3, ERR_WAIT_CHECK = 32, ERR_WAIT_SPLIT = 33 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -71,6 +71,15 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint32
             return false;
         }
     }
+}
+
+// mbar_wait for a converged warp whose lanes go on together: true in every lane or in none.  Near the time
+// limit lanes may disagree (one gives up, another's next poll succeeds), and a lane that went on
+// alone would wait for the others in the next warp-wide instruction (__syncwarp, tcgen05.ld) without any
+// limit.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, uint32_t* err, uint32_t code,
+                                               uint64_t limit_ns = kWaitLimitNs) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, err, code, limit_ns));
 }
 
 // Waits (bounded) for the phase whatever the error flag says: no copy may still be writing shared

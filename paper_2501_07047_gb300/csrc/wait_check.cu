@@ -33,7 +33,29 @@ __global__ void __launch_bounds__(32, 1) wait_check_kernel(uint32_t* err, uint64
     tc::tmem_dealloc(tmem, 32);
 }
 
+// The wait of a warp whose lanes go on together (tc::mbar_wait_warp): a lane whose bit of `lanes` is set
+// waits on a barrier that has completed, the others on one that nothing arrives on.  Lanes that
+// decide differently are recorded as tc::ERR_WAIT_SPLIT.
+__global__ void __launch_bounds__(32, 1) wait_check_warp_kernel(uint32_t* err, uint64_t limit_ns, uint32_t lanes) {
+    __shared__ uint64_t bar[2];
+    if (threadIdx.x == 0) {
+        tc::mbar_init(&bar[0], 1);
+        tc::mbar_init(&bar[1], 1);
+        tc::fence_mbar_init();
+        tc::mbar_arrive(&bar[1]);
+    }
+    __syncthreads();
+    const bool ok = tc::mbar_wait_warp(&bar[(lanes >> threadIdx.x) & 1u], 0, err, tc::ERR_WAIT_CHECK, limit_ns);
+    const uint32_t went_on = __ballot_sync(0xffffffffu, ok);
+    if (threadIdx.x == 0 && went_on != 0u && went_on != 0xffffffffu) atomicExch(err, (uint32_t)tc::ERR_WAIT_SPLIT);
+}
+
 }  // namespace
+
+cudaError_t launch_wait_check_warp(uint32_t* err, uint64_t limit_ns, uint32_t lanes, cudaStream_t s) {
+    wait_check_warp_kernel<<<1, 32, 0, s>>>(err, limit_ns, lanes);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_wait_check(uint32_t* err, uint64_t limit_ns, int arrive, cudaStream_t s) {
     wait_check_kernel<<<1, 32, 0, s>>>(err, limit_ns, arrive);

@@ -1,0 +1,43 @@
+"""Bounded waits of whole warps are decided for the whole warp: in the kernels whose roles run
+warp-wide instructions after a wait (tcgen05.ld, __syncwarp), a wait decided lane by lane is left
+to one elected thread, or its result is not used."""
+import pathlib
+import re
+
+import pytest
+
+CSRC = pathlib.Path(__file__).resolve().parent.parent / "paper_2501_07047_gb300" / "csrc"
+ELECTED = re.compile(r"if \((lane|tid|threadIdx\.x) == 0")
+
+
+def per_lane_decisions(source):
+    """Line numbers of tc::mbar_wait calls whose result decides something outside the block of an
+    elected thread."""
+    found, blocks, head = [], [], ""
+    for number, line in enumerate(source.splitlines(), 1):
+        code = line.split("//")[0]
+        if "tc::mbar_wait(" in code and not code.strip().startswith("tc::mbar_wait("):
+            if not any(ELECTED.search(b) for b in blocks) and not ELECTED.search(code):
+                found.append(number)
+        for ch in code:
+            if ch == "{":
+                blocks.append(head)
+                head = ""
+            elif ch == "}":
+                blocks.pop()
+                head = ""
+            elif ch == ";":
+                head = ""
+            else:
+                head += ch
+    return found
+
+
+def test_the_scan_sees_a_decision_by_lanes():
+    planted = "void k() {\n  if (lane == 0) {\n    if (!tc::mbar_wait(b)) return;\n  }\n  if (!tc::mbar_wait(b)) return;\n}\n"
+    assert per_lane_decisions(planted) == [5]
+
+
+@pytest.mark.parametrize("name", ["bconv_tc.cu"])
+def test_warps_decide_together(name):
+    assert per_lane_decisions((CSRC / name).read_text()) == []
