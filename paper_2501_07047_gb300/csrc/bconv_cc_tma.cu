@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(kThreads, HEFX_BCT_MINB)
     uint32_t it = 0;
     for (uint32_t t = blockIdx.x; t < ntiles; t += gridDim.x, ++it) {
         const uint32_t s = it % kStages, ph = (it / kStages) & 1u;
-        if (!tc::mbar_wait(&full[s], ph, err, tc::ERR_TIMEOUT_FULL)) break;
+        if (!tc::mbar_wait_warp(&full[s], ph, err, tc::ERR_TIMEOUT_FULL)) break;
         uint32_t* raw = reinterpret_cast<uint32_t*>(stage_raw) + (size_t)s * words + tid;
         const uint32_t b = t / tiles_per_poly, x = (t % tiles_per_poly) * kTile + tid;
         uint32_t* dst = out + ((size_t)b * Lp << log2n) + x;

@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(THREADS, 1) bat_ntt_gemm(const __grid_constant
         const uint32_t lq = (uint32_t)(warp - 4) * 32;
         const TcLimb lc = a.limbs[limb];
         for (uint32_t ob = 0; ob < n_ob; ++ob) {
-            if (!tc::mbar_wait(acc_full, ob & 1u, a.err, tc::ERR_TIMEOUT_ACC)) break;
+            if (!tc::mbar_wait_warp(acc_full, ob & 1u, a.err, tc::ERR_TIMEOUT_ACC)) break;
             tc::tc_fence_after();
             const uint32_t outi = ob * 128 + lq + lane;  // output index held by this thread
             for (int cb = 0; cb < NT; cb += 16) {

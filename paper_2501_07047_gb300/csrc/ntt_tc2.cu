@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             bool ok = true;
             for (uint32_t nt = 0; nt < ntiles; ++nt, ++t) {
                 const uint32_t acc = t & 1;
-                if (!tc::mbar_wait(&acc_full[acc], (t >> 1) & 1u, a.err, tc::ERR_TIMEOUT_ACC)) {
+                if (!tc::mbar_wait_warp(&acc_full[acc], (t >> 1) & 1u, a.err, tc::ERR_TIMEOUT_ACC)) {
                     ok = false;
                     break;
                 }

@@ -38,6 +38,6 @@ def test_the_scan_sees_a_decision_by_lanes():
     assert per_lane_decisions(planted) == [5]
 
 
-@pytest.mark.parametrize("name", ["bconv_tc.cu"])
+@pytest.mark.parametrize("name", ["bconv_tc.cu", "bconv_cc_tma.cu", "ntt_tc.cu", "ntt_tc2.cu"])
 def test_warps_decide_together(name):
     assert per_lane_decisions((CSRC / name).read_text()) == []
