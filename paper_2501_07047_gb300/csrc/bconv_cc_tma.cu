@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(kThreads, HEFX_BCT_MINB)
             }
             // no copy may still be writing shared memory when the CTA exits
             for (int s = 0; s < kStages; ++s)
-                if (issued[s]) tc::mbar_wait(&full[s], par[s], err, tc::ERR_TIMEOUT_FULL);
+                if (issued[s]) tc::mbar_drain(&full[s], par[s]);
         }
         return;
     }

@@ -349,7 +349,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
         if (leader) tc::mma_commit(mma_done);
         __syncwarp();
-        tc::mbar_wait(mma_done, 0, err, tc::ERR_TIMEOUT_ACC);
+        tc::mbar_drain(mma_done, 0);  // before TMEM is released, whatever the error flag says
     } else if (group < producers) {  // ---- step 1 and digits
         const uint32_t rx = (row & 7) << 4;
         Ring rr = {0, 0}, ra = {0, 0};

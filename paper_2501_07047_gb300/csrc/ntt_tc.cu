@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(THREADS, 1) bat_ntt_gemm(const __grid_constant
                     }
             // drain: every load this thread issued has landed before the CTA can exit
             for (int s = 0; s < STAGES; ++s)
-                if (issued[s]) tc::mbar_wait(&full[s], issued_parity[s], a.err, tc::ERR_TIMEOUT_FULL);
+                if (issued[s]) tc::mbar_drain(&full[s], issued_parity[s]);
         }
     } else if (warp == 1) {
         if (lane == 0) {  // ---- MMA issuer
@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(THREADS, 1) bat_ntt_gemm(const __grid_constant
             }
             // every MMA this thread issued has completed before TMEM is released
             tc::mma_commit(mma_done);
-            tc::mbar_wait(mma_done, 0, a.err, tc::ERR_TIMEOUT_ACC);
+            tc::mbar_drain(mma_done, 0);
         }
     } else if (warp >= 4) {  // ---- epilogue: one TMEM lane quadrant per warp
         const uint32_t lq = (uint32_t)(warp - 4) * 32;

@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(THREADS, 1)
 
     if (warp == 0) {
         if (lane == 0) {  // ---- TMA producer
-            uint32_t stage = 0, phase = 0;
+            uint32_t stage = 0, phase = 0, used = 0;
             bool ok = true;
             for (uint32_t item = cid; item < items && ok; item += nctas) {
                 uint32_t limb, poly0, drow0;
@@ -182,11 +182,21 @@ __global__ void __launch_bounds__(THREADS, 1)
                         tc::tma_load_2d(st, &amap, (int32_t)(kc * BK), (int32_t)a_row0, &full[stage]);
                         tc::tma_load_2d(st + A_BYTES, &bmap, (int32_t)(kc * BK), (int32_t)(b_row0 + nt * BN),
                                         &full[stage]);
+                        used = used < STAGES ? used + 1 : used;
                         if (++stage == STAGES) {
                             stage = 0;
                             phase ^= 1u;
                         }
                     }
+            }
+            // no copy may still be writing shared memory when the CTA exits (where the MMAs gave up)
+            for (uint32_t k = 0; k < used; ++k) {
+                if (stage == 0) {
+                    stage = STAGES;
+                    phase ^= 1u;
+                }
+                --stage;
+                tc::mbar_drain(&full[stage], phase);
             }
         }
     } else if (warp == 1) {
@@ -221,7 +231,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                     if (ok) tc::mma_commit(&acc_full[acc]);
                 }
             tc::mma_commit(mma_done);
-            tc::mbar_wait(mma_done, 0, a.err, tc::ERR_TIMEOUT_ACC);
+            tc::mbar_drain(mma_done, 0);  // before TMEM is released, whatever the error flag says
         }
     } else {  // ---- epilogue: warp % 4 is the TMEM lane quadrant, (warp - 2) / 4 the column slice
         const uint32_t quad = warp & 3, part = (warp - 2) >> 2;

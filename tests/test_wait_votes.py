@@ -1,6 +1,7 @@
 """Bounded waits of whole warps are decided for the whole warp: in the kernels whose roles run
 warp-wide instructions after a wait (tcgen05.ld, __syncwarp), a wait decided lane by lane is left
-to one elected thread, or its result is not used."""
+to one elected thread, or its result is not used.  What a kernel waits for before it ends (its
+copies and its MMAs) is waited for whatever the error flag says."""
 import pathlib
 import re
 
@@ -41,3 +42,12 @@ def test_the_scan_sees_a_decision_by_lanes():
 @pytest.mark.parametrize("name", ["bconv_tc.cu", "bconv_cc_tma.cu", "ntt_tc.cu", "ntt_tc2.cu"])
 def test_warps_decide_together(name):
     assert per_lane_decisions((CSRC / name).read_text()) == []
+
+
+@pytest.mark.parametrize("name", ["bconv_tc.cu", "bconv_cc_tma.cu", "ntt_tc.cu", "ntt_tc2.cu"])
+def test_last_waits_ignore_the_error_flag(name):
+    """tc::mbar_wait gives up as soon as another thread has; a wait whose result nobody uses is such a
+    last one and takes tc::mbar_drain."""
+    code = [line.split("//")[0].strip() for line in (CSRC / name).read_text().splitlines()]
+    assert [c for c in code if re.search(r"(^|\bif \(\w+\[\w+\]\) )tc::mbar_wait\(", c)] == []
+    assert any("tc::mbar_drain(" in c for c in code)
