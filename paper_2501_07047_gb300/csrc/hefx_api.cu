@@ -895,7 +895,7 @@ static cudaError_t batch_launch_all(hefx_batch_plan* plan, cudaStream_t s) {
         return launch_ntt_cc_batch(rows, static_cast<const BatchTask*>(plan->d_tasks), plan->ntasks, plan->off2,
                                    plan->err, s);
     for (const auto& l : plan->launches) {
-        cudaError_t e = launch_ntt_cc_rows(l.params, (NttMode)l.mode, rows + l.offset, l.nrows, s);
+        cudaError_t e = launch_ntt_cc_rows(l.params, l.params->max_prime, (NttMode)l.mode, rows + l.offset, l.nrows, s);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

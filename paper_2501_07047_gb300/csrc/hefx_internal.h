@@ -217,7 +217,8 @@ cudaError_t prepare_ntt_cc(const hefx_params* p, NttMode mode);
 // else the rescale kernel then the forward transform.
 cudaError_t launch_ntt_cc_rescale(const hefx_params* p, const uint32_t* in, uint32_t* out, size_t batch,
                                   cudaStream_t stream);
-cudaError_t launch_ntt_cc_rows(const hefx_params* p, NttMode mode, const RowDesc* d_rows, size_t nrows,
+// max_prime: the largest modulus of any row (rows may be of other parameter sets than p, at its N and schedule)
+cudaError_t launch_ntt_cc_rows(const hefx_params* p, uint32_t max_prime, NttMode mode, const RowDesc* d_rows, size_t nrows,
                                cudaStream_t stream);
 
 cudaError_t encode_input_map(const hefx_params* p, const uint32_t* in, size_t rows, CUtensorMap* map);

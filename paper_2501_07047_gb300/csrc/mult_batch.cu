@@ -259,7 +259,7 @@ hefx_status front_batch(hefx_ctx* ctx, hefx_mult_batch* mb, const hefx_mult_plan
     RowDesc* nttp = reinterpret_cast<RowDesc*>(hb + lay.nttp);
     MultRow* km = reinterpret_cast<MultRow*>(hb + lay.km);
     size_t q = 0, kmi = 0;
-    uint32_t lp_max = 0;
+    uint32_t lp_max = 0, max_q = 0;
     cudaError_t e = cudaSuccess;
     for (uint32_t r = 0; r < count && e == cudaSuccess; ++r) {
         MultPlanView v;
@@ -304,6 +304,7 @@ hefx_status front_batch(hefx_ctx* ctx, hefx_mult_batch* mb, const hefx_mult_plan
         bc[r].in = c;
         bc[r].out = pr;
         lp_max = std::max(lp_max, v.bc->Lp);
+        max_q = std::max(max_q, v.pq->max_prime);
         for (uint32_t j = 0; j < K; ++j) {
             nttp[(size_t)r * K + j] = rowdesc(pp, j, pr + j * n, pr + j * n);
             MultRow& k = km[kmi++];
@@ -325,11 +326,11 @@ hefx_status front_batch(hefx_ctx* ctx, hefx_mult_batch* mb, const hefx_mult_plan
         e = cudaGetLastError();
     }
     if (e == cudaSuccess)
-        e = launch_ntt_cc_rows(v0.pq, MODE_INV, reinterpret_cast<const RowDesc*>(db + lay.intt), r1, s);
+        e = launch_ntt_cc_rows(v0.pq, max_q, MODE_INV, reinterpret_cast<const RowDesc*>(db + lay.intt), r1, s);
     if (e == cudaSuccess)
         e = launch_bconv_cc_list(reinterpret_cast<const BcListEntry*>(db + lay.bc), count, logn, lp_max, s);
     if (e == cudaSuccess)
-        e = launch_ntt_cc_rows(pp, MODE_FWD, reinterpret_cast<const RowDesc*>(db + lay.nttp), (size_t)count * K, s);
+        e = launch_ntt_cc_rows(pp, pp->max_prime, MODE_FWD, reinterpret_cast<const RowDesc*>(db + lay.nttp), (size_t)count * K, s);
     if (e == cudaSuccess) {
         km_rows_kernel<<<grid_for(nkm << log2n4), 256, 0, s>>>(reinterpret_cast<const MultRow*>(db + lay.km),
                                                                (uint32_t)nkm, log2n4);

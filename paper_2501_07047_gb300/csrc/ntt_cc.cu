@@ -7,7 +7,9 @@
 
 namespace hefx {
 
-cudaError_t launch_dispatch(const hefx_params* p, NttMode mode, const cc::KArgs& a, size_t rows, cudaStream_t stream);
+// max_prime: the largest modulus of the rows, which decides between the lazy ranges (below 2^28) and Harvey's
+cudaError_t launch_dispatch(uint32_t log2n, uint32_t max_prime, NttMode mode, const cc::KArgs& a, size_t rows,
+                            cudaStream_t stream);
 
 namespace {
 
@@ -36,12 +38,13 @@ bool two_pass(const hefx_params* p, NttMode mode, size_t rows) {
     return (rows << p->log2n) >> 16 <= (mode == MODE_FWD ? 256u : mode == MODE_INV ? 320u : 144u);
 }
 
-cudaError_t launch_two_pass(const hefx_params* p, NttMode mode, const cc::KArgs& a, size_t rows, cudaStream_t stream) {
-    const bool lazy = p->max_prime < (1u << 28);
-    return p->log2n == 14 ? cc2::launch_14(mode, a, rows, stream, lazy)
-           : p->log2n == 15 ? cc2::launch_15(mode, a, rows, stream, lazy)
-           : p->log2n == 16 ? cc2::launch_16(mode, a, rows, stream, lazy)
-                            : cc2::launch_17(mode, a, rows, stream, lazy);
+cudaError_t launch_two_pass(uint32_t log2n, uint32_t max_prime, NttMode mode, const cc::KArgs& a, size_t rows,
+                            cudaStream_t stream) {
+    const bool lazy = max_prime < (1u << 28);
+    return log2n == 14 ? cc2::launch_14(mode, a, rows, stream, lazy)
+           : log2n == 15 ? cc2::launch_15(mode, a, rows, stream, lazy)
+           : log2n == 16 ? cc2::launch_16(mode, a, rows, stream, lazy)
+                         : cc2::launch_17(mode, a, rows, stream, lazy);
 }
 
 // The product's second half, INTT(NTT(b) o c) with c in the output, as the cluster forward transform
@@ -57,10 +60,10 @@ bool halves(const hefx_params* p, NttMode mode, size_t rows) {
 }
 
 cudaError_t launch_halves(const hefx_params* p, cc::KArgs& a, size_t rows, cudaStream_t stream) {
-    cudaError_t e = launch_dispatch(p, MODE_FWD_HAD, a, rows, stream);
+    cudaError_t e = launch_dispatch(p->log2n, p->max_prime, MODE_FWD_HAD, a, rows, stream);
     if (e != cudaSuccess) return e;
     a.in = a.out;
-    return launch_two_pass(p, MODE_INV_R, a, rows, stream);
+    return launch_two_pass(p->log2n, p->max_prime, MODE_INV_R, a, rows, stream);
 }
 
 }  // namespace
@@ -101,7 +104,7 @@ cudaError_t launch_ntt_cc(const hefx_params* p, NttMode mode, const uint32_t* in
     a.in_rows = 0;
     if (rows == 0) return cudaSuccess;
     if (halves(p, mode, rows)) return launch_halves(p, a, rows, stream);
-    return tp ? launch_two_pass(p, mode, a, rows, stream) : launch_dispatch(p, mode, a, rows, stream);
+    return tp ? launch_two_pass(p->log2n, p->max_prime, mode, a, rows, stream) : launch_dispatch(p->log2n, p->max_prime, mode, a, rows, stream);
 }
 
 cudaError_t launch_ntt_cc_rescale(const hefx_params* p, const uint32_t* in, uint32_t* out, size_t batch,
@@ -128,15 +131,15 @@ cudaError_t launch_ntt_cc_rescale(const hefx_params* p, const uint32_t* in, uint
     a.rows = (uint32_t)rows;
     a.L = L - 1;
     a.in_rows = L;
-    if (tp) return launch_two_pass(p, MODE_RS_FWD, a, rows, stream);
-    cudaError_t e = launch_dispatch(p, MODE_RS_FWD, a, rows, stream);
+    if (tp) return launch_two_pass(p->log2n, p->max_prime, MODE_RS_FWD, a, rows, stream);
+    cudaError_t e = launch_dispatch(p->log2n, p->max_prime, MODE_RS_FWD, a, rows, stream);
     if (e != cudaErrorNotSupported) return e;
     // not fused at this N: rescale into out, then the forward transform of its L - 1 limbs
     e = launch_rescale(p, in, out, batch, stream);
     if (e != cudaSuccess) return e;
     a.in = out;
     a.in_rows = 0;
-    return launch_dispatch(p, MODE_FWD, a, rows, stream);
+    return launch_dispatch(p->log2n, p->max_prime, MODE_FWD, a, rows, stream);
 }
 
 cudaError_t prepare_ntt_cc(const hefx_params* p, NttMode mode) {
@@ -144,10 +147,10 @@ cudaError_t prepare_ntt_cc(const hefx_params* p, NttMode mode) {
     cc::KArgs a = {};
     a.err = p->d_err_cc;
     a.desc = &dummy;  // selects the row-list kernels; rows == 0 sets attributes without launching
-    return launch_dispatch(p, mode, a, 0, nullptr);
+    return launch_dispatch(p->log2n, p->max_prime, mode, a, 0, nullptr);
 }
 
-cudaError_t launch_ntt_cc_rows(const hefx_params* p, NttMode mode, const RowDesc* d_rows, size_t nrows,
+cudaError_t launch_ntt_cc_rows(const hefx_params* p, uint32_t max_prime, NttMode mode, const RowDesc* d_rows, size_t nrows,
                                cudaStream_t stream) {
     cc::KArgs a;
     memset(&a.tmap_in, 0, sizeof a.tmap_in);
@@ -164,12 +167,14 @@ cudaError_t launch_ntt_cc_rows(const hefx_params* p, NttMode mode, const RowDesc
     a.L = p->nlimbs;
     a.in_rows = 0;
     if (nrows == 0) return cudaSuccess;
-    return two_pass(p, mode, nrows) ? launch_two_pass(p, mode, a, nrows, stream) : launch_dispatch(p, mode, a, nrows, stream);
+    return two_pass(p, mode, nrows) ? launch_two_pass(p->log2n, max_prime, mode, a, nrows, stream)
+                                    : launch_dispatch(p->log2n, max_prime, mode, a, nrows, stream);
 }
 
-cudaError_t launch_dispatch(const hefx_params* p, NttMode mode, const cc::KArgs& a, size_t rows, cudaStream_t stream) {
-    const bool lazy = p->max_prime < (1u << 28);
-    const int L = (int)p->log2n;
+cudaError_t launch_dispatch(uint32_t log2n, uint32_t max_prime, NttMode mode, const cc::KArgs& a, size_t rows,
+                            cudaStream_t stream) {
+    const bool lazy = max_prime < (1u << 28);
+    const int L = (int)log2n;
     if (L >= 3 && L <= 11) return cc::launch_range_a(L, mode, a, rows, stream, lazy);
     if (L >= 12 && L <= 14) return cc::launch_range_b(L, mode, a, rows, stream, lazy);
     if (L == 15) return cc::launch_range_c(L, mode, a, rows, stream, lazy);
