@@ -167,7 +167,8 @@ hefx_status hefx_params_set_reduction(hefx_params* params, hefx_reduction ntt_re
  *    blocks (reversed for the inverse); the intermediate goes through the output buffer.
  *  - HEFX_CC_AUTO (default): at N = 2^14 .. 2^17 the two-pass form while the intermediate stays
  *    in L2 (forward up to 256 rows of 2^16 elements, inverse 320, rescaling forward 144), and at
- *    N = 2^17, for the inverse at N = 2^16 and for that of a Hadamard product always; else
+ *    N = 2^17, for the inverse at N = 2^16 and for that of a Hadamard product always; else, and
+ *    for a hefx_ntt_fwd of at most 32 rows of 2^15 that is not captured into a graph,
  *    HEFX_CC_CLUSTER.
  * hefx_poly_mul's second half is the cluster forward transform, multiplying on its way out, and
  * the two-pass inverse unless HEFX_CC_CLUSTER is set (at N = 2^14 up to 128 rows); fused batch plans
@@ -176,6 +177,18 @@ hefx_status hefx_params_set_reduction(hefx_params* params, hefx_reduction ntt_re
  */
 typedef enum { HEFX_CC_AUTO = 0, HEFX_CC_CLUSTER = 1, HEFX_CC_TWO_PASS = 2 } hefx_cc_schedule;
 hefx_status hefx_params_set_cc_schedule(hefx_params* params, hefx_cc_schedule schedule);
+
+/*
+ * Kernel launches of one call on the CUDA-core path with the parameter set's present schedule:
+ * hefx_ntt_fwd, hefx_ntt_inv, hefx_ntt_inv_hadamard, hefx_rescale_ntt, or hefx_poly_mul of two
+ * different operands, on `batch` polynomials; captured != 0: on a stream that is being captured
+ * (a forward call of few rows of N = 2^15 is one launch otherwise).  0 for a null parameter set,
+ * an empty batch or an unknown form.
+ */
+typedef enum {
+    HEFX_FORM_FWD = 0, HEFX_FORM_INV = 1, HEFX_FORM_INV_HADAMARD = 2, HEFX_FORM_RESCALE_FWD = 3, HEFX_FORM_POLY_MUL = 4
+} hefx_ntt_form;
+uint32_t hefx_ntt_launches(const hefx_params* params, hefx_ntt_form form, size_t batch, int captured);
 
 /*
  * In-place forward NTT of d_data[batch][nlimbs][N] (natural order in, bit-reversed out).

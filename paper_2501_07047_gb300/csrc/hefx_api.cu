@@ -353,6 +353,27 @@ void hefx_params_destroy(hefx_params* p) {
     delete p;
 }
 
+// The legacy default stream cannot be captured (and must not be asked while another one is).
+static bool being_captured(cudaStream_t s) {
+    if (s == nullptr || s == cudaStreamLegacy) return false;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone;
+}
+
+uint32_t hefx_ntt_launches(const hefx_params* p, hefx_ntt_form form, size_t batch, int captured) {
+    if (!p || batch == 0) return 0;
+    const size_t rows = batch * p->nlimbs;
+    if (form == HEFX_FORM_FWD || form == HEFX_FORM_INV) {
+        const NttMode mode = form == HEFX_FORM_FWD ? MODE_FWD : MODE_INV;
+        return p->red_ntt != HEFX_RED_SHOUP ? 1u : ntt_cc_launches(p, mode, rows, !captured, false);
+    }
+    if (form == HEFX_FORM_INV_HADAMARD) return ntt_cc_launches(p, MODE_HAD_INV, rows, false, false);
+    if (form == HEFX_FORM_RESCALE_FWD) return ntt_cc_launches(p, MODE_RS_FWD, batch * (p->nlimbs - 1), false, false);
+    if (form != HEFX_FORM_POLY_MUL) return 0;
+    if (p->log2n <= 13) return 1;
+    return ntt_cc_launches(p, MODE_FWD, rows, false, false) + ntt_cc_launches(p, MODE_FWD_HAD_INV, rows, false, false);
+}
+
 static hefx_status run_ntt(hefx_ctx* ctx, const hefx_params* p, uint32_t* d, size_t batch, hefx_path path,
                            void* stream, NttMode mode) {
     hefx_status st = check_ntt_args(ctx, p, d, "d_data");
@@ -373,7 +394,9 @@ static hefx_status run_ntt(hefx_ctx* ctx, const hefx_params* p, uint32_t* d, siz
         if (e == cudaErrorNotSupported)
             return fail(ctx, HEFX_EUNSUPPORTED, "non-default NTT reduction is built for N = 2^16 only");
     } else if (pth == HEFX_PATH_CUDACORE) {
-        e = launch_ntt_cc(p, mode, d, nullptr, d, batch * p->nlimbs, (cudaStream_t)stream);
+        const size_t rows = batch * p->nlimbs;
+        const bool lone = one_launch_if_lone(p, mode, rows) && !being_captured((cudaStream_t)stream);
+        e = launch_ntt_cc(p, mode, d, nullptr, d, rows, (cudaStream_t)stream, lone);
     } else {
         return fail(ctx, HEFX_EINVAL, "unknown path %d", (int)path);
     }

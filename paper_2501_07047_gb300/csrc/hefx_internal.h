@@ -194,8 +194,12 @@ cudaError_t launch_pdl(void (*kern)(Params...), dim3 grid, dim3 block, size_t sm
 enum NttMode { MODE_FWD = 0, MODE_INV = 1, MODE_FWD_HAD_INV = 2, MODE_HAD_INV = 3, MODE_RS_FWD = 4, MODE_FWD_HAD = 5,
                MODE_INV_R = 6, MODE_PRODUCT = 7 };
 
+// lone: the call is this one transform, launched as it is made (not into a graph)
 cudaError_t launch_ntt_cc(const hefx_params* p, NttMode mode, const uint32_t* in, const uint32_t* had, uint32_t* out,
-                          size_t rows, cudaStream_t stream);
+                          size_t rows, cudaStream_t stream, bool lone = false);
+bool one_launch_if_lone(const hefx_params* p, NttMode mode, size_t rows);  // whether `lone` changes the schedule
+// The kernel launches of that (row_list: of launch_ntt_cc_rows).
+uint32_t ntt_cc_launches(const hefx_params* p, NttMode mode, size_t rows, bool lone, bool row_list);
 // Elementwise products of the HE-Mult request (elementwise.cu).
 cudaError_t launch_vec_mod_mul(const hefx_params* p, const uint32_t* x, const uint32_t* y, uint32_t* z, size_t rows,
                                cudaStream_t s);

@@ -29,11 +29,20 @@ namespace {
 //   inverse    9.3 / 6.3   26.0 / 20.5 44.6 / 36.8 60.7 / 57.3             22.0 / 14.8 62.2 / 43.7 219 / 170
 //   rescaling  9.3 / 6.7   27.8 / 24.0 45.7 / 44.0 63.1 / 64.9             19.5 / 16.4 56.3 / 52.6 209 / 196
 // and at N = 2^14 768 rows 43.1 / 38.3 and 40.8 / 34.3, 15 rows 7.9 / 5.0 and 8.7 / 5.2.
-bool two_pass(const hefx_params* p, NttMode mode, size_t rows) {
+//
+// A lone forward call (a call of its own, on a stream that is not being captured) of at most 32 rows of
+// 2^15 stays one cluster launch.  A launch costs the host 1.4 us, and a PyTorch program that looks its
+// current stream up for each call (2.8 us) is bound by the host with two of them: 8.5 us a call, 4
+// rows, against 7.4 with one.  Where the program keeps the stream the device decides, 4.7 against
+// 7.4 us, so captured calls, row lists and the halves of a product take two launches.  The other
+// forms and sizes are level or better with two either way (one / two launches, stream looked up:
+// N = 2^14 forward 8.5 / 8.5, inverse 8.7 / 8.6; 2^15 inverse 8.5 / 8.6).
+bool two_pass(const hefx_params* p, NttMode mode, size_t rows, bool lone = false) {
     if (p->log2n < 14 || p->log2n > 17 || mode == MODE_FWD_HAD_INV || mode == MODE_PRODUCT ||
         rows > (1u << 24))
         return false;
     if (p->cc_schedule != HEFX_CC_AUTO) return p->cc_schedule == HEFX_CC_TWO_PASS;
+    if (lone && mode == MODE_FWD && p->log2n == 15 && rows <= 32) return false;
     if (p->log2n == 17 || mode == MODE_HAD_INV || (p->log2n == 16 && mode == MODE_INV)) return true;
     return (rows << p->log2n) >> 16 <= (mode == MODE_FWD ? 256u : mode == MODE_INV ? 320u : 144u);
 }
@@ -78,12 +87,12 @@ cudaError_t encode_input_map(const hefx_params* p, const uint32_t* in, size_t ro
 }
 
 cudaError_t launch_ntt_cc(const hefx_params* p, NttMode mode, const uint32_t* in, const uint32_t* had, uint32_t* out,
-                          size_t rows, cudaStream_t stream) {
+                          size_t rows, cudaStream_t stream, bool lone) {
     cc::KArgs a;
     memset(&a.tmap_in, 0, sizeof a.tmap_in);
     memset(&a.tmap_out, 0, sizeof a.tmap_out);
     a.err = p->d_err_cc;
-    const bool tp = two_pass(p, mode, rows);
+    const bool tp = two_pass(p, mode, rows, lone);
     if (mode == MODE_INV && rows > 0 && p->log2n >= 13 && !tp) {
         cudaError_t e = encode_input_map(p, in, rows, &a.tmap_in);
         if (e != cudaSuccess) return e;
@@ -104,7 +113,19 @@ cudaError_t launch_ntt_cc(const hefx_params* p, NttMode mode, const uint32_t* in
     a.in_rows = 0;
     if (rows == 0) return cudaSuccess;
     if (halves(p, mode, rows)) return launch_halves(p, a, rows, stream);
-    return tp ? launch_two_pass(p->log2n, p->max_prime, mode, a, rows, stream) : launch_dispatch(p->log2n, p->max_prime, mode, a, rows, stream);
+    return tp ? launch_two_pass(p->log2n, p->max_prime, mode, a, rows, stream)
+              : launch_dispatch(p->log2n, p->max_prime, mode, a, rows, stream);
+}
+
+bool one_launch_if_lone(const hefx_params* p, NttMode mode, size_t rows) {
+    return two_pass(p, mode, rows) && !two_pass(p, mode, rows, true);
+}
+
+uint32_t ntt_cc_launches(const hefx_params* p, NttMode mode, size_t rows, bool lone, bool row_list) {
+    if (rows == 0) return 0;
+    if (!row_list && halves(p, mode, rows)) return 3;
+    if (mode == MODE_RS_FWD && p->log2n <= 13) return 2;  // rescaled, then transformed
+    return two_pass(p, mode, rows, lone) ? 2 : 1;
 }
 
 cudaError_t launch_ntt_cc_rescale(const hefx_params* p, const uint32_t* in, uint32_t* out, size_t batch,

@@ -34,7 +34,7 @@
 namespace hefx {
 namespace cc2 {
 
-using cc::KArgs;
+using cc::KRows;
 using cc::fwd_first;
 using cc::inv_offset;
 using cc::inv_sum;
@@ -203,7 +203,7 @@ __device__ __forceinline__ uint4 pack(const uint32_t (&x)[4]) { return make_uint
 
 // Forward in -> out (RS: rescaling on the way in), inverse in place in out.
 template <int LOGN, int MODE, int F, int SMALL>
-__device__ __forceinline__ void strided_task(uint2* tws, uint32_t* swap, uint32_t row, uint32_t part, const KArgs& a) {
+__device__ __forceinline__ void strided_task(uint2* tws, uint32_t* swap, uint32_t row, uint32_t part, const KRows& a) {
     typedef Strided<LOGN, SMALL> S;
     constexpr int N = 1 << LOGN, A = S::A, V = S::V, R = S::R, E = 1 << R, RA = 1 << A;
     constexpr bool INV = MODE == MODE_INV || MODE == MODE_HAD_INV, RS = MODE == MODE_RS_FWD;
@@ -306,7 +306,7 @@ __device__ __forceinline__ void load_tw_block(uint2 (&w)[31], uint32_t J, const 
 // place in out (canonical results), inverse in -> out (HAD: the Montgomery product of two inputs on
 // the way in).
 template <int LOGN, int MODE, int F>
-__device__ __forceinline__ void block_task(uint32_t* sm, uint32_t row, uint32_t blk, const KArgs& a) {
+__device__ __forceinline__ void block_task(uint32_t* sm, uint32_t row, uint32_t blk, const KRows& a) {
     constexpr int N = 1 << LOGN, A = LOGN - LOGB;
     constexpr bool INV = MODE == MODE_INV || MODE == MODE_HAD_INV, HAD = MODE == MODE_HAD_INV;
     const int lane = threadIdx.x & 31;
@@ -383,7 +383,7 @@ __device__ __forceinline__ void block_task(uint32_t* sm, uint32_t row, uint32_t 
 }
 
 template <int LOGN, int MODE, int F, int SMALL>
-__global__ void __launch_bounds__(THREADS, SM_WARPS * 32 / THREADS) strided_kernel(const __grid_constant__ KArgs a) {
+__global__ void __launch_bounds__(THREADS, SM_WARPS * 32 / THREADS) strided_kernel(const __grid_constant__ KRows a) {
     typedef Strided<LOGN, SMALL> S;
     __shared__ __align__(16) uint2 tws[1 << S::A];
     __shared__ uint32_t swap[S::SPLIT ? (1 << (S::R - 1)) * THREADS : 1];
@@ -392,7 +392,7 @@ __global__ void __launch_bounds__(THREADS, SM_WARPS * 32 / THREADS) strided_kern
 }
 
 template <int LOGN, int MODE, int F>
-__global__ void __launch_bounds__(32, SM_WARPS) block_kernel(const __grid_constant__ KArgs a) {
+__global__ void __launch_bounds__(32, SM_WARPS) block_kernel(const __grid_constant__ KRows a) {
     __shared__ __align__(16) uint32_t sm[BLOCK];
     constexpr uint32_t BLOCKS = (1u << LOGN) / BLOCK;
     griddep_wait();
@@ -400,7 +400,7 @@ __global__ void __launch_bounds__(32, SM_WARPS) block_kernel(const __grid_consta
 }
 
 template <int LOGN, int MODE, int F, int SMALL>
-cudaError_t launch_pair_t(const KArgs& a, size_t rows, cudaStream_t s) {
+cudaError_t launch_pair_t(const KRows& a, size_t rows, cudaStream_t s) {
     constexpr bool INV = MODE != MODE_FWD && MODE != MODE_RS_FWD;
     // the scale N^-1 2^32 is the strided pass's only difference, the product the block pass's
     constexpr int MS = MODE == MODE_INV_R ? MODE_HAD_INV : MODE, MB = MODE == MODE_INV_R ? MODE_INV : MODE;
@@ -421,7 +421,7 @@ cudaError_t launch_pair_t(const KArgs& a, size_t rows, cudaStream_t s) {
 //   inverse    6.4 / 5.2  6.9 / 5.7  9.5 / 8.7  13.6 / 13.2  39.5 / 39.0  81.1 / 83.8
 //   rescaling             7.6 / 6.0  10.2/ 9.3  14.6 / 13.3  47.0 / 45.7  92.9 / 87.8
 template <int LOGN, int MODE, int F>
-cudaError_t launch_pair(const KArgs& a, size_t rows, cudaStream_t s) {
+cudaError_t launch_pair(const KRows& a, size_t rows, cudaStream_t s) {
     constexpr bool RS = MODE == MODE_RS_FWD;
     const size_t rows16 = (rows << LOGN) >> 16;
     if constexpr (LOGN == 17) return launch_pair_t<LOGN, MODE, F, 0>(a, rows, s);
@@ -432,7 +432,7 @@ cudaError_t launch_pair(const KArgs& a, size_t rows, cudaStream_t s) {
 
 // rows == 0 launches nothing
 template <int LOGN, int F>
-cudaError_t launch_mode(NttMode mode, const KArgs& a, size_t rows, cudaStream_t s) {
+cudaError_t launch_mode(NttMode mode, const KRows& a, size_t rows, cudaStream_t s) {
     switch (mode) {
         case MODE_FWD: return launch_pair<LOGN, MODE_FWD, F>(a, rows, s);
         case MODE_INV: return launch_pair<LOGN, MODE_INV, F>(a, rows, s);
@@ -447,17 +447,17 @@ cudaError_t launch_mode(NttMode mode, const KArgs& a, size_t rows, cudaStream_t 
 
 // lazy: every modulus of the parameter set is below 2^28
 template <int LOGN>
-cudaError_t launch_logn(NttMode mode, const KArgs& a, size_t rows, cudaStream_t s, bool lazy) {
+cudaError_t launch_logn(NttMode mode, const KRows& a, size_t rows, cudaStream_t s, bool lazy) {
     if (rows == 0) return cudaSuccess;
     if (a.desc) return lazy ? launch_mode<LOGN, 3>(mode, a, rows, s) : launch_mode<LOGN, 1>(mode, a, rows, s);
     return lazy ? launch_mode<LOGN, 2>(mode, a, rows, s) : launch_mode<LOGN, 0>(mode, a, rows, s);
 }
 
 // One ring degree each, compiled in its own translation unit (build time).
-cudaError_t launch_14(NttMode mode, const KArgs& a, size_t rows, cudaStream_t s, bool lazy);
-cudaError_t launch_15(NttMode mode, const KArgs& a, size_t rows, cudaStream_t s, bool lazy);
-cudaError_t launch_16(NttMode mode, const KArgs& a, size_t rows, cudaStream_t s, bool lazy);
-cudaError_t launch_17(NttMode mode, const KArgs& a, size_t rows, cudaStream_t s, bool lazy);
+cudaError_t launch_14(NttMode mode, const KRows& a, size_t rows, cudaStream_t s, bool lazy);
+cudaError_t launch_15(NttMode mode, const KRows& a, size_t rows, cudaStream_t s, bool lazy);
+cudaError_t launch_16(NttMode mode, const KRows& a, size_t rows, cudaStream_t s, bool lazy);
+cudaError_t launch_17(NttMode mode, const KRows& a, size_t rows, cudaStream_t s, bool lazy);
 
 }  // namespace cc2
 }  // namespace hefx

@@ -4,7 +4,7 @@
 namespace hefx {
 namespace cc2 {
 
-cudaError_t launch_14(NttMode mode, const KArgs& a, size_t rows, cudaStream_t s, bool lazy) {
+cudaError_t launch_14(NttMode mode, const KRows& a, size_t rows, cudaStream_t s, bool lazy) {
     return launch_logn<14>(mode, a, rows, s, lazy);
 }
 

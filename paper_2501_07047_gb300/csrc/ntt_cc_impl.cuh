@@ -148,11 +148,8 @@ struct Cfg {
     static_assert(threads >= 128, "at least four warps per CTA");
 };
 
-struct KArgs {
-    // the input viewed as [rows * N / 32][32] uint32, 128-byte swizzle, box 32 x 256: the
-    // inverse transforms of the contiguous layout load their part of a row with it (TMA)
-    alignas(64) CUtensorMap tmap_in;
-    CUtensorMap tmap_out;  // the output, same view: forward transforms store their part with it
+// What a transform kernel is given; the two-pass kernels take this alone.
+struct KRows {
     uint32_t* err;      // bounded-wait error flag (a device word, 0 = no error)
     const uint32_t* in;
     const uint32_t* had;
@@ -167,6 +164,13 @@ struct KArgs {
     uint32_t in_rows;  // MODE_RS_FWD: input rows per polynomial (the output has L = in_rows - 1)
 };
 
+struct KArgs : KRows {
+    // the input viewed as [rows * N / 32][32] uint32, 128-byte swizzle, box 32 x 256: the
+    // inverse transforms of the contiguous layout load their part of a row with it (TMA)
+    alignas(64) CUtensorMap tmap_in;
+    CUtensorMap tmap_out;  // the output, same view: forward transforms store their part with it
+};
+
 // Flag bits of F in the one-launch product (MODE_PRODUCT): operands are written earlier in the same
 // launch; and its second half, whose input is a.had and whose Hadamard operand is a.out.
 constexpr int kFresh = 128, kSecond = 256;
@@ -175,17 +179,17 @@ constexpr int kFresh = 128, kSecond = 256;
 // is one, else from the contiguous [batch][L][N] layout.
 // F is a compile-time switch so that the contiguous-layout kernels carry no descriptor code.
 template <int N, int F>
-__device__ __forceinline__ const uint32_t* row_in(const KArgs& a, uint32_t r) {
+__device__ __forceinline__ const uint32_t* row_in(const KRows& a, uint32_t r) {
     if constexpr ((F & 1) != 0) return a.desc[r].in;
     else return ((F & kSecond) != 0 ? a.had : a.in) + (size_t)r * N;
 }
 template <int N, int F>
-__device__ __forceinline__ const uint32_t* row_had(const KArgs& a, uint32_t r) {
+__device__ __forceinline__ const uint32_t* row_had(const KRows& a, uint32_t r) {
     if constexpr ((F & 1) != 0) return a.desc[r].had;
     else return ((F & kSecond) != 0 ? a.out : a.had) + (size_t)r * N;
 }
 template <int N, int F>
-__device__ __forceinline__ uint32_t* row_out(const KArgs& a, uint32_t r) {
+__device__ __forceinline__ uint32_t* row_out(const KRows& a, uint32_t r) {
     if constexpr ((F & 1) != 0) return a.desc[r].out;
     else return a.out + (size_t)r * N;
 }
@@ -198,17 +202,17 @@ __device__ __forceinline__ uint32_t row_limb(const KArgs& a, uint32_t r) {
 // parameter set's tables, so rows of different ring degrees can share a launch), else from the
 // launch's parameter set.
 template <int F>
-__device__ __forceinline__ const LimbConst& row_lc(const KArgs& a, uint32_t r) {
+__device__ __forceinline__ const LimbConst& row_lc(const KRows& a, uint32_t r) {
     if constexpr ((F & 1) != 0) return *a.desc[r].lc;
     else return a.lc[r % a.L];
 }
 template <int N, int F>
-__device__ __forceinline__ const uint2* row_twf(const KArgs& a, uint32_t r) {
+__device__ __forceinline__ const uint2* row_twf(const KRows& a, uint32_t r) {
     if constexpr ((F & 1) != 0) return a.desc[r].twf;
     else return a.tw_f + (size_t)(r % a.L) * N;
 }
 template <int N, int F>
-__device__ __forceinline__ const uint2* row_twi(const KArgs& a, uint32_t r) {
+__device__ __forceinline__ const uint2* row_twi(const KRows& a, uint32_t r) {
     if constexpr ((F & 1) != 0) return a.desc[r].twi;
     else return a.tw_i + (size_t)(r % a.L) * N;
 }

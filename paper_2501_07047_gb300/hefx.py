@@ -44,6 +44,7 @@ SIGNATURES = {
     "hefx_basis_convert": (_i32, [_vp, _vp, _vp, _vp, _sz, _i32, _vp]),
     "hefx_stream_check": (_i32, [_vp, _vp, _vp]),
     "hefx_wait_check": (_i32, [_vp, _vp, ctypes.c_uint64, _i32, _vp]),
+    "hefx_ntt_launches": (_u32, [_vp, _i32, _sz, _i32]),
     "hefx_wait_check_warp": (_i32, [_vp, _vp, ctypes.c_uint64, _u32, _vp]),
     "hefx_vec_mod_mul": (_i32, [_vp, _vp, _vp, _vp, _vp, _sz, _vp]),
     "hefx_tensor_product": (_i32, [_vp, _vp, _vp, _vp, _vp, _vp, _vp, _vp, _vp, _sz, _vp]),
@@ -189,6 +190,14 @@ def hefx_params_set_tensor_config(ctx, params: int, log2r: int = 0, tile_outputs
     """Tensor-path split (N = 2^log2r x rest, or with log2r2 > 0 the three factors 2^log2r x
     2^log2r2 x rest; log2r = 0: the square two-factor split) and GEMM tile width."""
     _check(ctx, load().hefx_params_set_tensor_config(params, int(log2r), int(log2r2), int(tile_outputs)))
+
+
+NTT_FORMS = {"fwd": 0, "inv": 1, "inv_hadamard": 2, "rescale_fwd": 3, "poly_mul": 4}
+
+
+def hefx_ntt_launches(params: int, form: str, batch: int, captured: bool = False) -> int:
+    """Kernel launches of one CUDA-core call of `form` (see include/hefx.h)."""
+    return int(load().hefx_ntt_launches(params, NTT_FORMS[form], batch, int(bool(captured))))
 
 
 def hefx_ntt_fwd(ctx, params, data, batch, path="cudacore", stream=None) -> None:
