@@ -870,13 +870,13 @@ def tensor_split(log2r: int = 0, log2r2: int = 0):
 
 def profile_traffic(kernel: str, which: str):
     """DRAM bytes per launch of the `which` ("fwd" / "inv") kernel from the committed ncu
-    summary, if it matches the current source."""
+    summary, if it matches the current source (the file or comma-separated files it names)."""
     path = os.path.join(ROOT, "profiles", f"{kernel}_traffic.txt")
     try:
         kv = dict(ln.split("=", 1) for ln in open(path).read().split("\n") if "=" in ln)
         import hashlib
-        src = os.path.join(ROOT, "paper_2501_07047_gb300", "csrc", kv["source"].strip())
-        if hashlib.sha256(open(src, "rb").read()).hexdigest()[:16] != kv["source_sha"].strip():
+        src = [os.path.join(ROOT, "paper_2501_07047_gb300", "csrc", s.strip()) for s in kv["source"].split(",")]
+        if hashlib.sha256(b"".join(open(s, "rb").read() for s in src)).hexdigest()[:16] != kv["source_sha"].strip():
             return None
         return int(float(kv["dram_bytes_per_launch_" + which]))
     except Exception:

@@ -49,7 +49,7 @@ using cc::twmul;
 
 constexpr int LOGB = 10, BLOCK = 1 << LOGB;  // elements of a block
 
-constexpr int SM_WARPS = 20;                 // warps an SM that the register budget is sized for (102 registers)
+constexpr int SM_WARPS = 20;                 // warps an SM that the register budget is sized for (96 registers)
 
 // Twiddles g, g + 1 of a stage (base in shared memory, 16-byte aligned for even g).
 __device__ __forceinline__ void tw_pair(uint2 (&w)[2], const uint2* base) {
@@ -292,7 +292,7 @@ __device__ __forceinline__ void strided_task(uint2* tws, uint32_t* swap, uint32_
 __device__ __forceinline__ uint4* chunk_of(uint32_t* sm, int e) { return reinterpret_cast<uint4*>(&sm[cc::swz(e)]); }
 
 // Twiddles of inverse stages E0 .. E1-1 of sub-transform J over 32 consecutive elements (as
-// cc::load_tw_inv): requested in two parts, the first with the data, which 102 registers allow.
+// cc::load_tw_inv): requested in two parts, the first with the data, which 96 registers allow.
 template <int LOGN, int E0, int E1>
 __device__ __forceinline__ void load_tw_block(uint2 (&w)[31], uint32_t J, const uint2* tw) {
 #pragma unroll
