@@ -302,10 +302,14 @@ hefx_status hefx_bconv_check(hefx_ctx* ctx, const hefx_bconv_plan* plan, void* s
  * [batch][L][N] and d_U [batch][dnum][L + K][N], coefficient form, canonical, 16-byte aligned;
  * d_U must not overlap d_c (EINVAL).  hefx_modup_check waits for `stream` and reports and clears
  * an expired bounded wait of the plan's launches, as hefx_bconv_check does for conversions.
+ * hefx_modup_plan_set_path(HEFX_PATH_CUDACORE) keeps the plan's ModUps on the CUDA cores
+ * (HEFX_PATH_AUTO, the default, decides as above; other paths EINVAL; not thread-safe with
+ * concurrent calls that use the plan).
  */
 hefx_status hefx_modup_plan_create(hefx_ctx* ctx, uint32_t log2n, const uint32_t* q, uint32_t L, const uint32_t* p,
                                    uint32_t K, uint32_t alpha, hefx_modup_plan** out);
 void hefx_modup_plan_destroy(hefx_modup_plan* plan);
+hefx_status hefx_modup_plan_set_path(hefx_modup_plan* plan, hefx_path path);
 uint32_t hefx_modup_plan_dnum(const hefx_modup_plan* plan); /* 0 for a null plan */
 hefx_status hefx_mod_up(hefx_ctx* ctx, const hefx_modup_plan* plan, const uint32_t* d_c, uint32_t* d_U, size_t batch,
                         void* stream);
@@ -362,9 +366,13 @@ hefx_status hefx_key_inner_product(hefx_ctx* ctx, const hefx_params* params, con
  * special limbs) and d_out is [batch][L][N].  The conversion is the fast one of
  * hefx_basis_convert, so the result represents floor(X / P) - u, 0 <= u < K, for the
  * integer X that d_x represents.  d_out must not overlap d_x.  Takes the path that
- * HEFX_PATH_AUTO gives the plan's conversion (hefx_bconv_check reports its waits).
+ * HEFX_PATH_AUTO gives the plan's conversion (hefx_bconv_check reports its waits), unless
+ * hefx_bconv_plan_set_mod_down_path(HEFX_PATH_CUDACORE) keeps the plan's ModDowns, this and
+ * hefx_mod_down_scaled, on the CUDA cores (HEFX_PATH_AUTO undoes it; other paths EINVAL; not
+ * thread-safe with concurrent calls that use the plan).
  * Errors: EINVAL for a null, foreign or misaligned argument or overlap.
  */
+hefx_status hefx_bconv_plan_set_mod_down_path(hefx_bconv_plan* plan, hefx_path path);
 hefx_status hefx_mod_down(hefx_ctx* ctx, const hefx_bconv_plan* plan, const uint32_t* d_x, uint32_t* d_out,
                           size_t batch, void* stream);
 

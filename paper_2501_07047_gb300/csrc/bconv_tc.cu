@@ -684,7 +684,7 @@ cudaError_t launch_bconv_tc(const hefx_bconv_plan* plan, const uint32_t* in, uin
 
 cudaError_t launch_mod_down_tc(const hefx_bconv_plan* plan, const uint32_t* x, uint32_t* out, size_t batch,
                                bool scaled, cudaStream_t stream) {
-    if (!bconv_prefer_tc(plan, batch) || plan->tc->small_target) return cudaErrorNotSupported;
+    if (plan->mod_down_cc || !bconv_prefer_tc(plan, batch) || plan->tc->small_target) return cudaErrorNotSupported;
     BcTcArgs a = {};
     a.out = out;
     a.xq = x;
@@ -700,7 +700,7 @@ cudaError_t launch_mod_down_tc(const hefx_bconv_plan* plan, const uint32_t* x, u
 
 cudaError_t launch_mod_up_tc(const hefx_modup_plan* mp, const uint32_t* c, uint32_t* U, size_t batch,
                              cudaStream_t stream) {
-    if (!bconv_tc_engine(mp->tc, mp->log2n) || mp->tc->small_target ||
+    if (mp->cc || !bconv_tc_engine(mp->tc, mp->log2n) || mp->tc->small_target ||
         !faster_on_tc(mp->alpha, mp->L + mp->K - mp->alpha, (batch * mp->dnum << mp->log2n) / TILE))
         return cudaErrorNotSupported;
     BcTcArgs a = {};

@@ -547,6 +547,21 @@ void hefx_modup_plan_destroy(hefx_modup_plan* mp) {
     delete mp;
 }
 
+static hefx_status fused_path(hefx_ctx* ctx, hefx_path path, bool* cc) {
+    if (path != HEFX_PATH_AUTO && path != HEFX_PATH_CUDACORE)
+        return fail(ctx, HEFX_EINVAL, "path must be HEFX_PATH_AUTO or HEFX_PATH_CUDACORE, not %d", (int)path);
+    *cc = path == HEFX_PATH_CUDACORE;
+    return HEFX_OK;
+}
+
+hefx_status hefx_modup_plan_set_path(hefx_modup_plan* mp, hefx_path path) {
+    return mp ? fused_path(mp->ctx, path, &mp->cc) : HEFX_EINVAL;
+}
+
+hefx_status hefx_bconv_plan_set_mod_down_path(hefx_bconv_plan* p, hefx_path path) {
+    return p ? fused_path(p->ctx, path, &p->mod_down_cc) : HEFX_EINVAL;
+}
+
 uint32_t hefx_modup_plan_dnum(const hefx_modup_plan* mp) { return mp ? mp->dnum : 0; }
 
 hefx_status hefx_mod_up(hefx_ctx* ctx, const hefx_modup_plan* plan, const uint32_t* c, uint32_t* U, size_t batch,

@@ -144,6 +144,7 @@ struct hefx_bconv_plan {
     std::vector<uint32_t> src, dst;
     void* d_const = nullptr;          // BConvConst (see bconv.cu)
     hefx::BcTcPlan* tc = nullptr;     // tensor form, null where it does not apply
+    bool mod_down_cc = false;         // ModDown stays on the CUDA cores (hefx_bconv_plan_set_mod_down_path)
     uint32_t* d_err = nullptr;        // bounded-wait error flag of the pipelined kernels (0 = none)
 };
 
@@ -155,6 +156,7 @@ struct hefx_modup_plan {
     std::vector<uint32_t> q, p;
     void* d_const = nullptr;  // dnum BConvConst
     hefx::BcTcPlan* tc = nullptr;  // tensor form of every digit, null where it does not apply
+    bool cc = false;               // ModUp stays on the CUDA cores (hefx_modup_plan_set_path)
     uint32_t* d_err = nullptr;     // its bounded-wait error flag (0 = none)
 };
 

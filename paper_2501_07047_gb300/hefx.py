@@ -57,6 +57,8 @@ SIGNATURES = {
     "hefx_key_inner_product_add": (_i32, [_vp, _vp, _vp, _vp, _vp, _vp, _vp, _u32, _sz, _vp]),
     "hefx_modup_plan_create": (_i32, [_vp, _u32, _u32p, _u32, _u32p, _u32, _u32, ctypes.POINTER(_vp)]),
     "hefx_modup_plan_destroy": (None, [_vp]),
+    "hefx_modup_plan_set_path": (_i32, [_vp, _i32]),
+    "hefx_bconv_plan_set_mod_down_path": (_i32, [_vp, _i32]),
     "hefx_modup_plan_dnum": (_u32, [_vp]),
     "hefx_mod_up": (_i32, [_vp, _vp, _vp, _vp, _sz, _vp]),
     "hefx_modup_check": (_i32, [_vp, _vp, _vp]),
@@ -294,6 +296,16 @@ def hefx_modup_plan_create(ctx: int, log2n: int, q, p, alpha: int) -> int:
 
 def hefx_modup_plan_destroy(plan: int) -> None:
     load().hefx_modup_plan_destroy(plan)
+
+
+def hefx_modup_plan_set_path(ctx: int, plan: int, path="auto") -> None:
+    """"cudacore" keeps the plan's ModUps on the CUDA cores; "auto" takes the faster path."""
+    _check(ctx, load().hefx_modup_plan_set_path(plan, _path(path)))
+
+
+def hefx_bconv_plan_set_mod_down_path(ctx: int, plan: int, path="auto") -> None:
+    """"cudacore" keeps the plan's ModDowns on the CUDA cores; "auto" takes the faster path."""
+    _check(ctx, load().hefx_bconv_plan_set_mod_down_path(plan, _path(path)))
 
 
 def hefx_modup_plan_dnum(plan: int) -> int:

@@ -49,8 +49,9 @@ class HeMult:
         self.pQr = hefx.hefx_params_create(ctx, logn, self.qs[:-1])
         self.pQP = hefx.hefx_params_create(ctx, logn, self.qs + self.ps)
         qp = self.qs + self.ps
-        # ModUp: one launch for every digit on the CUDA cores ("auto", "cudacore"), or two
-        # conversions per digit through hefx_basis_convert on the requested path
+        # ModUp: one launch for every digit ("auto": on the faster path; "cudacore": on the CUDA
+        # cores, and ModDown too), or two conversions per digit through hefx_basis_convert on the
+        # requested path
         self.modup = hefx.hefx_modup_plan_create(ctx, logn, self.qs, self.ps, alpha) \
             if bconv_path in ("auto", "cudacore") else None
         self.plans = []
@@ -60,6 +61,9 @@ class HeMult:
             hi_plan = hefx.hefx_bconv_plan_create(ctx, logn, src, qp[hi:])
             self.plans.append((lo_plan, hi_plan))
         self.plan_pq = hefx.hefx_bconv_plan_create(ctx, logn, self.ps, self.qs)
+        if bconv_path == "cudacore":
+            hefx.hefx_modup_plan_set_path(ctx, self.modup, bconv_path)
+            hefx.hefx_bconv_plan_set_mod_down_path(ctx, self.plan_pq, bconv_path)
         n, L, K = 1 << logn, self.L, self.K
         dev = "cuda"
         self.d = torch.empty((3, L, n), dtype=torch.int32, device=dev)
