@@ -765,6 +765,7 @@ def bench_he_mult(ctx, args):
                                    "rescale_us": round(resc_ms * 1e3, 1), "K": alpha,
                                    "launches_he_mult": hm.launches(rescale=False),
                                    "launches_rescale": 2}  # rescale() alone: INTT, Rescale + NTT
+        hm.check(s)  # no bounded wait expired in any of these runs
         del g
         hm.close()
         del ins, evk, cq, out, cw

@@ -85,6 +85,26 @@ class HeMult:
         for p in (self.pQ, self.pQr, self.pQP):
             hefx.hefx_params_destroy(p)
 
+    def check(self, stream=None) -> None:
+        """Waits for `stream` (the current one by default) and raises HefxError(ETIMEOUT) if a bounded
+        device wait of an earlier run expired: of a conversion (ModUp, ModDown) or of a transform.  The
+        results of those runs are invalid; the record is cleared."""
+        st = self.torch.cuda.current_stream() if stream is None else stream
+        checks = [(hefx.hefx_modup_check, self.modup)] if self.modup else []
+        checks += [(hefx.hefx_bconv_check, p) for pair in self.plans for p in pair if p]
+        checks += [(hefx.hefx_bconv_check, self.plan_pq)]
+        checks += [(hefx.hefx_stream_check, p) for p in (self.pQ, self.pQr, self.pQP)]
+        expired = None
+        for check, handle in checks:  # all of them, so that every record is cleared
+            try:
+                check(self.ctx, handle, st)
+            except hefx.HefxError as e:
+                if e.status != hefx.HEFX_ETIMEOUT:
+                    raise
+                expired = expired or e
+        if expired:
+            raise expired
+
     def launches(self, rescale: bool = True) -> int:
         """Kernel launches of one run (CUDA-core NTT path)."""
         modup = 1 if self.modup else sum(2 if lo else 1 for lo, _ in self.digits)
