@@ -764,7 +764,7 @@ def bench_he_mult(ctx, args):
         res[f"L{L}_dnum{dnum}"] = {"he_mult_us": round(mult_ms * 1e3, 1), "he_mult_graph_us": round(graph_ms * 1e3, 1),
                                    "rescale_us": round(resc_ms * 1e3, 1), "K": alpha,
                                    "launches_he_mult": hm.launches(rescale=False),
-                                   "launches_rescale": 2}  # rescale() alone: INTT, Rescale + NTT
+                                   "launches_rescale": hm.rescale_launches()}
         hm.check(s)  # no bounded wait expired in any of these runs
         del g
         hm.close()

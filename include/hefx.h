@@ -608,8 +608,7 @@ hefx_status hefx_batch_plan_create(hefx_ctx* ctx, const hefx_job* jobs, size_t n
 void hefx_batch_plan_destroy(hefx_batch_plan* plan);
 
 /*
- * Transform launches one hefx_batch_polymul of the plan makes (1 for the fused form; a transform
- * on the two-pass schedule counts once).
+ * Kernel launches one hefx_batch_polymul of the plan makes (1 for the fused form).
  */
 uint32_t hefx_batch_plan_launches(const hefx_batch_plan* plan);
 

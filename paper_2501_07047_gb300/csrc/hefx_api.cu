@@ -924,7 +924,9 @@ void hefx_batch_plan_destroy(hefx_batch_plan* plan) {
 uint32_t hefx_batch_plan_launches(const hefx_batch_plan* plan) {
     if (!plan) return 0;
     if (plan->fused) return plan->ntasks ? 1u : 0u;
-    return (uint32_t)plan->launches.size();
+    uint32_t n = 0;
+    for (const auto& l : plan->launches) n += ntt_cc_launches(l.params, (NttMode)l.mode, l.nrows, false, true);
+    return n;
 }
 
 static cudaError_t batch_launch_all(hefx_batch_plan* plan, cudaStream_t s) {

@@ -105,10 +105,20 @@ class HeMult:
         if expired:
             raise expired
 
-    def launches(self, rescale: bool = True) -> int:
-        """Kernel launches of one run (CUDA-core NTT path)."""
-        modup = 1 if self.modup else sum(2 if lo else 1 for lo, _ in self.digits)
-        return 1 + 1 + modup + 1 + 1 + 1 + 1 + (1 if rescale else 2)
+    def launches(self, rescale: bool = True, captured: bool = False) -> int:
+        """Kernel launches of one run (CUDA-core NTT path), eager or captured into a graph."""
+        def count(params, form, batch):
+            return hefx.hefx_ntt_launches(params, form, batch, captured)
+
+        n = 1 + count(self.pQ, "inv_hadamard", 1)  # tensor product, INTT(a1 o b1)
+        n += 1 if self.modup else sum(2 if lo else 1 for lo, _ in self.digits)
+        n += count(self.pQP, "fwd", self.dnum) + 1 + count(self.pQP, "inv", 2) + 1  # .., inner product, .., ModDown
+        return n + (count(self.pQ, "rescale_fwd", 2) if rescale else count(self.pQ, "fwd", 2) + 1)
+
+    def rescale_launches(self, captured: bool = False) -> int:
+        """Kernel launches of rescale() (CUDA-core NTT path)."""
+        return (hefx.hefx_ntt_launches(self.pQ, "inv", 2, captured) +
+                hefx.hefx_ntt_launches(self.pQ, "rescale_fwd", 2, captured))
 
     def run(self, a0, a1, b0, b1, evk, out, stream=None, rescale: bool = True) -> None:
         """a*, b*: [L][N] evaluation form over Q; evk: [dnum][2][L+K][N] evaluation form over
@@ -158,7 +168,7 @@ class HeMult:
     def rescale(self, c, out, stream=None) -> None:
         """c: [2][L][N] evaluation form over Q (overwritten) -> out [2][L-1][N] evaluation form
         over q_0 .. q_{L-2}: NTT(Rescale(INTT(c))); on the CUDA-core path the rescale runs on
-        the forward transform's input load (two launches)."""
+        the forward transform's input load."""
         st = self.torch.cuda.current_stream() if stream is None else stream
         with self.torch.cuda.stream(st):
             hefx.hefx_ntt_inv(self.ctx, self.pQ, c, 2, self.ntt_path, st)
