@@ -2,8 +2,9 @@
 and records the fastest as what HEFX_PATH_AUTO runs.
 
 Candidates (all bit-exact; checked by INTT(NTT(x)) = x before timing):
-  - the CUDA-core radix-2 path, under each of its schedules at N = 2^16 (one launch of 8-CTA
-    clusters, or the two-pass column / block schedule; `hefx_params_set_cc_schedule`);
+  - the CUDA-core radix-2 path, under each of its schedules (`hefx_params_set_cc_schedule`): at
+    N = 2^16 one launch of 8-CTA clusters or the two-pass schedule; at 2^14, 2^15 and 2^17 the
+    library's own choice (two-pass for most row counts) or the clusters;
   - the tensor-core matrix NTT for every valid two-factor split N = R x C and the three-factor
     splits R1 x R2 x R3 with the fewest digit MACs (`tensor_plan.tuned_splits`: the paper sweeps
     its (R, C) configurations per operator and keeps the best, Sec. V-A), each with both GEMM
@@ -59,18 +60,24 @@ def candidates(logn: int) -> list:
     return out
 
 
+def alternatives(logn: int) -> list:
+    """CUDA-core schedules beside the library's own choice, timed after the candidates: the cluster
+    schedule where that choice is the two-pass one and cannot be named."""
+    return [("cudacore", 1, 0, 0)] if logn in (14, 15, 17) else []
+
+
 def apply(ctx: int, params: int, cand) -> None:
     path, log2r, log2r2, tile = cand
     if path == "tensor":
         hefx.hefx_params_set_tensor_config(ctx, params, log2r, tile, log2r2)
-    else:
-        hefx.hefx_params_set_cc_schedule(ctx, params, CC_SCHEDULES[log2r])
+    # explicit CUDA-core calls keep the library's choice where the tensor path wins
+    hefx.hefx_params_set_cc_schedule(ctx, params, CC_SCHEDULES[0 if path == "tensor" else log2r])
     hefx.hefx_params_set_auto_path(params, path)
 
 
-def time_candidates(ctx: int, params: int, logn: int, primes, batch: int = 4, reps: int = 5) -> dict:
-    """Median ms of one forward + inverse NTT of [batch][L][N] per available candidate, keyed
-    "path/log2r/log2r2/tile"."""
+def time_candidates(ctx: int, params: int, logn: int, primes, batch: int = 4, reps: int = 5, cands=None) -> dict:
+    """Median ms of one forward + inverse NTT of [batch][L][N] per available candidate (of
+    `candidates(logn)` unless given), keyed "path/log2r/log2r2/tile"."""
     import torch
     n = 1 << logn
     data = inputs.residue_tensor(inputs.derive_seed(90, logn, len(primes)), batch, primes, n)
@@ -78,7 +85,7 @@ def time_candidates(ctx: int, params: int, logn: int, primes, batch: int = 4, re
     d = d0.clone()
     s = torch.cuda.current_stream()
     out = {}
-    for cand in candidates(logn):
+    for cand in candidates(logn) if cands is None else cands:
         path = cand[0]
         if hefx.raw_status("hefx_ntt_fwd", ctx, params, d.data_ptr(), 0, hefx.PATHS[path], s.cuda_stream) != 0:
             continue
@@ -127,8 +134,9 @@ def tune(ctx: int, params: int, logn: int, primes, batch: int = 4, use_cache: bo
         best = cache[key]["config"]
     else:
         times = time_candidates(ctx, params, logn, primes, batch)
-        best = min(times, key=times.get)
-        cache[key] = {"config": best, "ms": times}
+        other = time_candidates(ctx, params, logn, primes, batch, cands=alternatives(logn)) if alternatives(logn) else {}
+        best = min({**times, **other}, key={**times, **other}.get)
+        cache[key] = {"config": best, "ms": times, "alternatives": other}
         if use_cache:
             _save_cache(cache)
     cand = parse(best)
