@@ -195,13 +195,15 @@ class HeMult:
             self.run(a0, a1, b0, b1, evk, out, torch.cuda.current_stream(), rescale)
         return g
 
-    def stages(self) -> dict:
+    def stages(self, rescale: bool | None = None) -> dict:
         """The workspaces after a run (for stage-by-stage parity tests).  The merged form keeps
         t (P^-1 acc + d over Q, acc over P) and c in coefficient form; the stages that it does not
-        compute are worked out from those here."""
+        compute are worked out from those here.  rescale: whether what ran last was with the Rescale
+        (after a graph's replay: as it was captured); by default as the last call of run()."""
         torch = self.torch
+        merged = self.merged if rescale is None else rescale and self.ntt_path == "cudacore"
         st = {"d0": self.d[0], "d1": self.d[1], "d2_coeff": self.c, "modup_eval": self.U, "c_coeff": self.cc}
-        if not self.merged:
+        if not merged:
             return {**st, "acc_coeff": self.acc, "ks_eval": self.ks}
         s = torch.cuda.current_stream()
         q = torch.tensor(self.qs, dtype=torch.int64, device="cuda")[None, :, None]
