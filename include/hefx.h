@@ -161,7 +161,7 @@ hefx_status hefx_params_set_reduction(hefx_params* params, hefx_reduction ntt_re
  * return identical results.
  *  - HEFX_CC_CLUSTER: one launch; a row of N = 2^16 is split over a cluster of 8 CTAs and
  *    its three cross-CTA stages go through distributed shared memory.
- *  - HEFX_CC_TWO_PASS (N = 2^16 only): two launches through L2, the row / column
+ *  - HEFX_CC_TWO_PASS (to be asked for at N = 2^16 only): two launches through L2, the row / column
  *    factorisation of the matrix NTT (Sec. IV-B) with the twiddle step folded into the
  *    butterflies: log2 N - 10 stages over elements 1024 apart, then 10 within 1024-element
  *    blocks (reversed for the inverse); the intermediate goes through the output buffer.
@@ -169,11 +169,16 @@ hefx_status hefx_params_set_reduction(hefx_params* params, hefx_reduction ntt_re
  *    in L2 (forward up to 256 rows of 2^16 elements, inverse 320, rescaling forward 144), and at
  *    N = 2^17, for the inverse at N = 2^16 and for that of a Hadamard product always; else, and
  *    for a hefx_ntt_fwd of at most 32 rows of 2^15 that is not captured into a graph,
- *    HEFX_CC_CLUSTER.
+ *    HEFX_CC_CLUSTER.  These lines hold for a GPU that runs one transform at a time.  Where
+ *    independent batches overlap on several streams their intermediates no longer share L2, and
+ *    the clusters' partial last wave fills with the other stream's: 192 rows of 2^16 a call, forward
+ *    and inverse, 5.27 M limb-NTT/s with AUTO against 5.39 M with HEFX_CC_CLUSTER on two streams (one
+ *    call at a time 4.33 M against 3.85 M).  A program of that kind sets HEFX_CC_CLUSTER.
  * hefx_poly_mul's second half is the cluster forward transform, multiplying on its way out, and
- * the two-pass inverse unless HEFX_CC_CLUSTER is set (at N = 2^14 up to 128 rows); fused batch plans
- * use the cluster schedule.  Errors:
- * EINVAL (unknown schedule), EUNSUPPORTED (HEFX_CC_TWO_PASS at N != 2^16).  Not thread-safe with concurrent calls that use the same params.
+ * the two-pass inverse unless HEFX_CC_CLUSTER is set (at N = 2^14 up to 128 rows); fused batch
+ * plans use the cluster schedule.
+ * Errors: EINVAL (unknown schedule), EUNSUPPORTED (HEFX_CC_TWO_PASS at N != 2^16).  Not thread-safe
+ * with concurrent calls that use the same params.
  */
 typedef enum { HEFX_CC_AUTO = 0, HEFX_CC_CLUSTER = 1, HEFX_CC_TWO_PASS = 2 } hefx_cc_schedule;
 hefx_status hefx_params_set_cc_schedule(hefx_params* params, hefx_cc_schedule schedule);

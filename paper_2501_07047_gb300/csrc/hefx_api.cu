@@ -1136,7 +1136,7 @@ hefx_status hefx_params_set_cc_schedule(hefx_params* p, hefx_cc_schedule schedul
     if (schedule != HEFX_CC_AUTO && schedule != HEFX_CC_CLUSTER && schedule != HEFX_CC_TWO_PASS)
         return fail(p->ctx, HEFX_EINVAL, "unknown CUDA-core schedule %d", (int)schedule);
     if (schedule == HEFX_CC_TWO_PASS && p->log2n != 16)
-        return fail(p->ctx, HEFX_EUNSUPPORTED, "the two-pass schedule is built for N = 2^16 only");
+        return fail(p->ctx, HEFX_EUNSUPPORTED, "HEFX_CC_TWO_PASS can be asked for at N = 2^16 only (HEFX_CC_AUTO takes it at 2^14 .. 2^17)");
     p->cc_schedule = (int)schedule;
     return HEFX_OK;
 }

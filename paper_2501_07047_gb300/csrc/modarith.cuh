@@ -19,7 +19,7 @@ __device__ __forceinline__ uint32_t mul_shoup_lazy(uint32_t x, uint32_t w, uint3
     return x * w - quot * q;
 }
 
-// Montgomery REDC of x * y (x < 4q, y < q): returns x y 2^-32 mod q in [0, 2q).
+// Montgomery REDC of x * y (any x < 2^32, y < q, so x y < q 2^32): returns x y 2^-32 mod q in [0, 2q).
 __device__ __forceinline__ uint32_t mul_mont_lazy(uint32_t x, uint32_t y, uint32_t q, uint32_t qinv_neg) {
     uint64_t z = (uint64_t)x * y;
     uint32_t lo = (uint32_t)z, hi = (uint32_t)(z >> 32);
